@@ -70,7 +70,9 @@ typedef struct {
                               <= 0 means 64 * d * 2^-53                                         */
     double collapse_tol;   /* RD_MIXED: reject when two roots lie within collapse_tol * max(1,|z|) */
     int32_t block;         /* threads per CTA, multiple of 32 in [32, 256] (up to 512 with
-                              polish_warps > 0, see below); 0 = the default                  */
+                              polish_warps > 0, see below); 0 = the default. With block,
+                              ctas_per_sm, lanes, polish_warps and ring_slots all 0 the library
+                              picks the form as well (by degree and n; same roots bit for bit) */
     int32_t ctas_per_sm;   /* grid = ctas_per_sm x SM count; 0 = tuned default                   */
     int32_t polish_extra;  /* RD_MIXED: further Newton steps, p and p' both in FP64, for a root
                               that fails the residual check after polish_steps (0..16)          */
@@ -275,7 +277,9 @@ int rd_pointer_is_device_accessible(const void *p);
  * and joined back to `stream` with events, so the whole call can be captured
  * in a CUDA graph (as two parallel branches) and `stream` orders everything
  * before and after it. The first call on a device from a host thread creates
- * the helper stream and its two events; make that call outside capture. */
+ * the helper stream and its two events; make that call outside capture.
+ * (With the launch shape open -- no tuning, no shape in params -- a small batch
+ * is solved without bins, in 3 launches on `stream` and no helper stream.) */
 typedef struct {
     /* Launch shape of each degree bin's solve kernel, indexed by the degree
      * (entries 1..12; entries 0 and 13..15 are ignored). 0 = the default.   */

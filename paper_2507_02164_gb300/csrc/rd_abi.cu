@@ -30,7 +30,9 @@ int l2_nodes_host(int nr, double *r, double *w);
 size_t uneven_workspace_bytes(int64_t n, int64_t n_coeffs, rd_dtype dt);
 int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const int64_t *offsets, int64_t n,
                   int64_t n_coeffs, bool mixed, void *ws, const int *block, const int *cps, const int *lanes,
-                  const int *pw, bool fork, cudaStream_t st);
+                  const int *pw, bool fork, bool open_shape, cudaStream_t st);
+bool group_takes(int degree, int64_t n, bool mixed);
+int launch_group(int degree, rd_dtype dt, bool mixed, const SolveArgs &a, cudaStream_t st);
 int launch_l2(const double *samples, int64_t n, int nr, int degree, double *coeffs, int precision,
               cudaStream_t st);
 int roots_uneven_common(const void *coeffs, rd_dtype dtype, const uint8_t *degrees, const int64_t *offsets, int64_t n,
@@ -130,6 +132,12 @@ int check_params(const rd_params &p)
     return RD_OK;
 }
 
+// The caller left the whole launch shape to the library.
+bool shape_open(const rd_params &p)
+{
+    return p.block == 0 && p.ctas_per_sm == 0 && p.lanes == 0 && p.polish_warps == 0 && p.ring_slots == 0;
+}
+
 // Validate a tile clip (host struct, device arrays) for n polynomials.
 int check_clip(const rd_clip &c, int64_t n)
 {
@@ -212,6 +220,8 @@ int solve_common(const void *coeffs, rd_dtype dtype, int degree, int64_t n, rd_m
     a.n = n;
     if (n == 0) return RD_OK;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if (shape_open(p) && rd::group_takes(degree, n, mode == RD_MIXED))
+        return rd::launch_group(degree, dtype, mode == RD_MIXED, a, st);
     if (p.polish_warps > 0) {
         if (mode != RD_MIXED) return rd_set_error(RD_EINVAL, "params.polish_warps > 0 needs RD_MIXED");
         return rd::launch_solve_ws(degree, dtype, a, p.block, p.ctas_per_sm, p.polish_warps, p.ring_slots, st);
@@ -433,7 +443,7 @@ int roots_uneven_common(const void *coeffs, rd_dtype dtype, const uint8_t *degre
     a.coeffs = coeffs;
     a.n = n;
     return rd::launch_uneven(a, dtype, degrees, offsets, n, n_coeffs, mode == RD_MIXED, ws, block, cps, lanes, pw,
-                             fork, reinterpret_cast<cudaStream_t>(stream));
+                             fork, !tuning && shape_open(p), reinterpret_cast<cudaStream_t>(stream));
 }
 
 }  // namespace rd

@@ -262,34 +262,41 @@ __device__ __forceinline__ dfl two_prod(float a, float b)
 // FP32 point x for coefficients a_k = hi_k + lo_k (lo only when LO). Each
 // Horner step's product acc * x and sum with hi_k are split error-free into
 // a float and its rounding error (four TwoProducts, four TwoSums); the errors
-// run through a second Horner recurrence. On return p + err equals p(x) as
-// if evaluated in twice the working precision, and d1 = p'(x), d2 = p''(x)/2
-// in FP32 (plain Horner on the FP32 iterates). TwoProduct and TwoSum are
+// run through a second Horner recurrence. After the last step P + E equals
+// p(x) as if evaluated in twice the working precision, and D1 = p'(x), D2 =
+// p''(x)/2 in FP32 (plain Horner on the FP32 iterates). TwoProduct and TwoSum are
 // error-free, so their outputs do not depend on how the real operations are
 // grouped; the plain sums of the errors keep the scalar order per part. The
 // same bits as the scalar form, about 35 instead of 50 issue slots per
 // coefficient (one-role compensated polish on the degree-6 Littlewood batch
 // 16 % faster).
-template <int N, bool LO>
-__device__ __forceinline__ void comp_horner(const cx<float> (&hi)[N + 1], const cx<float> (&lo)[LO ? N + 1 : 1],
-                                            cx<float> x, cx<float> &p, cx<float> &err, cx<float> &d1,
-                                            cx<float> &d2)
-{
-    // On (real, imaginary) pairs as packed FP32 instructions, each half the
-    // scalar scheme's operation on that part (a product with -x_im is the
-    // negated product exactly), in one issue slot for both:
-    //   a z = (a_re x_re - a_im x_im, a_re x_im + a_im x_re)
-    //       = bcast(a_re) (x_re, x_im) + bcast(a_im) (-x_im, x_re)
-    const float2 X = make_float2(x.re, x.im), Xr = make_float2(-x.im, x.re);
-    auto bc = [](float v) { return make_float2(v, v); };
-    auto neg2 = [](float2 v) { return make_float2(-v.x, -v.y); };
-    // a z + c, as cfma
-    auto cfma2 = [&](float2 a, float2 c) { return __ffma2_rn(bc(a.x), X, __ffma2_rn(bc(a.y), Xr, c)); };
-    float2 P = make_float2(hi[N].re, hi[N].im);
-    float2 E = LO ? make_float2(lo[LO ? N : 0].re, lo[LO ? N : 0].im) : make_float2(0.0f, 0.0f);
-    float2 D1 = make_float2(0.0f, 0.0f), D2 = make_float2(0.0f, 0.0f);
-#pragma unroll
-    for (int k = N - 1; k >= 0; --k) {
+struct CompHorner {
+    float2 X, Xr;          // (x_re, x_im), (-x_im, x_re)
+    float2 P, E, D1, D2;   // iterate, its error, p', p''/2
+
+    static __device__ __forceinline__ float2 bc(float v) { return make_float2(v, v); }
+    static __device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
+    // a x + c, as cfma
+    __device__ __forceinline__ float2 cfma2(float2 a, float2 c) const
+    {
+        return __ffma2_rn(bc(a.x), X, __ffma2_rn(bc(a.y), Xr, c));
+    }
+    // start at the leading coefficient hi + lo
+    __device__ __forceinline__ CompHorner(cx<float> x, cx<float> hi, cx<float> lo)
+    {
+        X = make_float2(x.re, x.im);
+        Xr = make_float2(-x.im, x.re);
+        P = make_float2(hi.re, hi.im);
+        E = make_float2(lo.re, lo.im);
+        D1 = D2 = make_float2(0.0f, 0.0f);
+    }
+    // the next coefficient down. On (real, imaginary) pairs as packed FP32
+    // instructions, each half the scalar scheme's operation on that part (a
+    // product with -x_im is the negated product exactly), in one issue slot
+    // for both: a z = bcast(a_re) (x_re, x_im) + bcast(a_im) (-x_im, x_re)
+    template <bool LO>
+    __device__ __forceinline__ void step(cx<float> hi, cx<float> lo)
+    {
         D2 = cfma2(D2, D1);
         D1 = cfma2(D1, P);
         // (t1, t3) = p_re (x_re, x_im), (-t2, t4) = p_im (-x_im, x_re), each with its exact error
@@ -299,20 +306,33 @@ __device__ __forceinline__ void comp_horner(const cx<float> (&hi)[N + 1], const 
         const float2 S = __fadd2_rn(Ah, Bh);
         const float2 Sb = __fadd2_rn(S, neg2(Ah));
         const float2 Se = __fadd2_rn(__fadd2_rn(Ah, neg2(__fadd2_rn(S, neg2(Sb)))), __fadd2_rn(Bh, neg2(Sb)));
-        const float2 H = make_float2(hi[k].re, hi[k].im);
+        const float2 H = make_float2(hi.re, hi.im);
         const float2 U = __fadd2_rn(S, H);
         const float2 Ub = __fadd2_rn(U, neg2(S));
         const float2 Ue = __fadd2_rn(__fadd2_rn(S, neg2(__fadd2_rn(U, neg2(Ub)))), __fadd2_rn(H, neg2(Ub)));
         P = U;
         float2 Er = __fadd2_rn(__fadd2_rn(__fadd2_rn(Al, Bl), Se), Ue);
-        if constexpr (LO) Er = __fadd2_rn(Er, make_float2(lo[k].re, lo[k].im));
+        if constexpr (LO) Er = __fadd2_rn(Er, make_float2(lo.re, lo.im));
         E = cfma2(E, Er);
     }
-    p = {P.x, P.y};
-    err = {E.x, E.y};
-    d1 = {D1.x, D1.y};
-    d2 = {D2.x, D2.y};
-}
+    // One Newton step of z = zh + zl (zh = x): p(z) = p(zh) + p'(zh) zl +
+    // p''(zh)/2 zl^2, step p(z)/p'(zh) in FP32, z <- z - dz by TwoSum on the
+    // high parts, then renormalised. false: the step is not finite, z stays.
+    __device__ __forceinline__ bool newton(cx<float> &zh, cx<float> &zl) const
+    {
+        const cx<float> d1 = {D1.x, D1.y}, d2 = {D2.x, D2.y};
+        const cx<float> corr = mul(cfma(d2, zl, d1), zl);
+        const cx<float> r = {__fadd_rn(P.x, __fadd_rn(E.x, corr.re)), __fadd_rn(P.y, __fadd_rn(E.y, corr.im))};
+        const cx<float> dz = cdiv(r, d1);
+        if (!(isfinite(dz.re) && isfinite(dz.im))) return false;
+        const dfl sr = two_sum(zh.re, -dz.re), si = two_sum(zh.im, -dz.im);
+        const dfl nr = fast_two_sum(sr.hi, __fadd_rn(sr.lo, zl.re));
+        const dfl ni = fast_two_sum(si.hi, __fadd_rn(si.lo, zl.im));
+        zh = {nr.hi, ni.hi};
+        zl = {nr.lo, ni.lo};
+        return true;
+    }
+};
 
 // Split d * 2^-shift into hi + lo floats (|d * 2^-shift| <= 2): hi = d's
 // significand rounded to 24 bits, lo = the rest rounded to 24 bits (relative

@@ -1,0 +1,79 @@
+// rd_group.cu -- launches of the small-batch solver (rd_group.cuh) and the
+// sizes that take it.
+#include "rd_group.cuh"
+
+namespace rd {
+
+// Whether a uniform batch takes the small-batch solver when the caller left
+// the launch shape open. Measured (us, 152 SMs, group / one thread per
+// polynomial at 32 threads per CTA, one launch with binning):
+//   mixed, n   700: degree 3 14.6 / 16.7   6 33.0 / 51.4   12  76.0 / 186.7
+//             4800: degree 3 16.5 / 16.5   6 35.1 / 45.4   12 110.8 / 190.8
+//             6000: degree 3 16.5 / 16.7   9 86.3 / 92.5   12 127.9 / 192.9
+//             8000: degree 3 18.6 / 16.6   9  125 / 86.2   12 186.5 / 190.9
+//   plain, n  1216: degree 5  250 / 234    6  338 / 347    12  1179 / 1972
+//             2432: degree 5  250 / 225    6  367 / 361    12  1847 / 1908
+// so the line lies at 40 polynomials per SM (mixed, from degree 3) and at 8
+// (plain, from degree 6: its FP64 instructions cost the same for one active
+// lane as for 32).
+bool group_takes(int degree, int64_t n, bool mixed)
+{
+    const int64_t sms = rd_sm_count_cached();
+    return mixed ? degree >= 3 && n <= 40 * sms : degree >= 6 && n <= 8 * sms;
+}
+
+// The same for a packed batch of mixed degrees, which this solver takes in
+// one launch after the count, where the degree bins are twelve kernels on two
+// chains, each as long as its slowest warp. Measured (us, degrees 2..12,
+// complex128, group / bins): mixed 1000 97 / 484, 3001 109 / 483, 16000
+// 249 / 521, 32000 415 / 556, 64000 753 / 643; plain 1000 1023 / 4198, 8000
+// 4081 / 6027, 16000 7435 / 6960.
+bool uneven_group_takes(int64_t n, bool mixed) { return n <= (int64_t)(mixed ? 256 : 64) * rd_sm_count_cached(); }
+
+template <int G, typename In, int MODE>
+static int launch_group_n(int degree, const SolveArgs &a, cudaStream_t st)
+{
+    constexpr int P = 32 / G;
+    solve_group_kernel<G, In, MODE><<<(unsigned)((a.n + P - 1) / P), GROUP_BLOCK, 0, st>>>(a, degree);
+    return rd_check_launch("solve_group_kernel");
+}
+
+template <int G, typename In>
+static int launch_group_mode(int degree, bool mixed, const SolveArgs &a, cudaStream_t st)
+{
+    if (!mixed) return launch_group_n<G, In, MODE_PLAIN>(degree, a, st);
+    if (a.polish_mode == RD_POLISH_DF) return launch_group_n<G, In, MODE_MIXED_DF>(degree, a, st);
+    return launch_group_n<G, In, MODE_MIXED_FP64>(degree, a, st);
+}
+
+int launch_group(int degree, rd_dtype dt, bool mixed, const SolveArgs &a, cudaStream_t st)
+{
+    if (degree <= 8)
+        return dt == RD_C64 ? launch_group_mode<8, float2>(degree, mixed, a, st)
+                            : launch_group_mode<8, double2>(degree, mixed, a, st);
+    return dt == RD_C64 ? launch_group_mode<16, float2>(degree, mixed, a, st)
+                        : launch_group_mode<16, double2>(degree, mixed, a, st);
+}
+
+template <typename In>
+static int launch_uneven_group_mode(const SolveArgs &a, const UnevenArgs &U, const UnevenHeader *hdr, bool mixed,
+                                    cudaStream_t st)
+{
+    const unsigned grid = (unsigned)((U.n + 1) / 2);
+    if (!mixed)
+        uneven_group_kernel<In, MODE_PLAIN><<<grid, GROUP_BLOCK, 0, st>>>(a, U, hdr);
+    else if (a.polish_mode == RD_POLISH_DF)
+        uneven_group_kernel<In, MODE_MIXED_DF><<<grid, GROUP_BLOCK, 0, st>>>(a, U, hdr);
+    else
+        uneven_group_kernel<In, MODE_MIXED_FP64><<<grid, GROUP_BLOCK, 0, st>>>(a, U, hdr);
+    return rd_check_launch("uneven_group_kernel");
+}
+
+int launch_uneven_group(const SolveArgs &a, rd_dtype dt, const UnevenArgs &U, const UnevenHeader *hdr, bool mixed,
+                        cudaStream_t st)
+{
+    return dt == RD_C64 ? launch_uneven_group_mode<float2>(a, U, hdr, mixed, st)
+                        : launch_uneven_group_mode<double2>(a, U, hdr, mixed, st);
+}
+
+}  // namespace rd

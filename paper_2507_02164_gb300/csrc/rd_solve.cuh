@@ -123,19 +123,22 @@ __device__ __forceinline__ bool finite_c(cx<T> z) { return isfinite(z.re) && isf
 // residual test, but keeps the FP32 copies used for p'(z) and the residual
 // bound finite when coefficients lie beyond the FP32 range (an L2 fit of
 // sin(z^3) reaches 1e41). The exponents are read from the bits (integer ops).
+__device__ __forceinline__ unsigned exponent_bits(double v) { return ((unsigned)__double2hiint(v) >> 20) & 0x7ffu; }
+
+__device__ __forceinline__ double pow2_scale(unsigned emax)
+{
+    int sh = (int)emax - 1023;
+    sh = sh > 1000 ? 1000 : (sh < -1000 ? -1000 : sh);
+    return __longlong_as_double((long long)(1023 - sh) << 52);  // 2^-sh
+}
+
 template <int K>
 __device__ __forceinline__ void scale_pow2(cx<double> (&a)[K])
 {
     unsigned emax = 0;
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const unsigned er = ((unsigned)__double2hiint(a[k].re) >> 20) & 0x7ffu;
-        const unsigned ei = ((unsigned)__double2hiint(a[k].im) >> 20) & 0x7ffu;
-        emax = max(emax, max(er, ei));
-    }
-    int sh = (int)emax - 1023;
-    sh = sh > 1000 ? 1000 : (sh < -1000 ? -1000 : sh);
-    const double f = __longlong_as_double((long long)(1023 - sh) << 52);  // 2^-sh
+    for (int k = 0; k < K; ++k) emax = max(emax, max(exponent_bits(a[k].re), exponent_bits(a[k].im)));
+    const double f = pow2_scale(emax);
 #pragma unroll
     for (int k = 0; k < K; ++k) a[k] = {a[k].re * f, a[k].im * f};
 }
@@ -457,8 +460,8 @@ __device__ __forceinline__ void sweep_lane(const SolveArgs &A, const void *coeff
 // caller's tighter rtol, NaN. Measured (one role, bit for bit the same): 2^26
 // degree-6 Littlewood polynomials 90.1 -> 76.5 ms, 100,003 of degree 12 828 ->
 // 718 us, 2^22 of degrees 2..12 10.98 -> 9.46 ms.
-template <int N>
-__device__ __forceinline__ bool residual_certain(float dz1, float drift, float az, float den, float lead, float rtol)
+__device__ __forceinline__ bool residual_certain(int N, float dz1, float drift, float az, float den, float lead,
+                                                 float rtol)
 {
     return dz1 < (0x1p-31f / N) * az && drift <= 0x1p-20f * az && az >= 0x1p-60f && az <= 0x1p60f &&
            den >= 0x1p-60f && den <= 0x1p60f && lead >= 0x1p-100f && rtol >= 63.9999f * N * 0x1p-53f;
@@ -531,6 +534,7 @@ __device__ __forceinline__ void finish_lane(const SolveArgs &A, const void *coef
                 // complex64 coefficients are exact in FP32 and have none
                 constexpr bool LO = MODE == MODE_MIXED_DF && !std::is_same<In, float2>::value;
                 cx<float> alo[LO ? N + 1 : 1];
+                if constexpr (!LO) alo[0] = {0.0f, 0.0f};
                 if constexpr (LO) {
 #pragma unroll
                     for (int k = 0; k <= N; ++k)
@@ -565,19 +569,10 @@ __device__ __forceinline__ void finish_lane(const SolveArgs &A, const void *coef
                         // the step size in FP32
                         cx<float> zl = {0.0f, 0.0f};
                         for (int step = 0; step < A.polish_steps; ++step) {
-                            cx<float> p, err, d1, d2;
-                            comp_horner<N, LO>(af, alo, zf, p, err, d1, d2);
-                            const cx<float> corr = mul(cfma(d2, zl, d1), zl);
-                            const cx<float> r = {__fadd_rn(p.re, __fadd_rn(err.re, corr.re)),
-                                                 __fadd_rn(p.im, __fadd_rn(err.im, corr.im))};
-                            const cx<float> dz = cdiv(r, d1);
-                            if (!finite_c(dz)) break;
-                            // z <- z - dz: TwoSum on the high parts, then renormalise
-                            const dfl sr = two_sum(zf.re, -dz.re), si = two_sum(zf.im, -dz.im);
-                            const dfl nr = fast_two_sum(sr.hi, __fadd_rn(sr.lo, zl.re));
-                            const dfl ni = fast_two_sum(si.hi, __fadd_rn(si.lo, zl.im));
-                            zf = {nr.hi, ni.hi};
-                            zl = {nr.lo, ni.lo};
+                            CompHorner ch(zf, af[N], alo[LO ? N : 0]);
+#pragma unroll
+                            for (int k = N - 1; k >= 0; --k) ch.step<LO>(af[k], alo[LO ? k : 0]);
+                            if (!ch.newton(zf, zl)) break;
                             newton += 1;
                         }
                         // zh + zl rounded once to FP64
@@ -610,7 +605,7 @@ __device__ __forceinline__ void finish_lane(const SolveArgs &A, const void *coef
                     if constexpr (MODE != MODE_MIXED_DF) {
                         const cx<float> zr = d2f(zj);
                         const float az = sqrtf(norm2(zr));
-                        good = residual_certain<N>(moved, abs1(sub(zr, zf)), az, weight(az), abs1(af[N]), rtol);
+                        good = residual_certain(N, moved, abs1(sub(zr, zf)), az, weight(az), abs1(af[N]), rtol);
                     }
                     if (!__all_sync(0xffffffffu, good || degenerate)) {
                         cx<double> p = ad[N];

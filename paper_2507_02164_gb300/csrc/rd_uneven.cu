@@ -20,40 +20,6 @@ namespace rd {
 
 int launch_clear(uint32_t *p, int64_t words, cudaStream_t st);
 
-
-struct UnevenArgs {
-    const uint8_t *degrees;
-    const int64_t *offsets;
-    int64_t n;
-    int64_t n_coeffs;
-};
-
-// A polynomial is solvable when its offsets hold exactly degree + 1
-// coefficients, its degree is 1..12, and its roots fit the packed root array
-// of n_coeffs - n elements: o0 >= i keeps root 0 (at o0 - i) at or above 0,
-// o1 <= n_coeffs - (n - 1 - i) keeps its last root (at o1 - i - 2) below
-// n_coeffs - n. The comparisons are ordered so that no difference overflows.
-// These bounds hold for each polynomial alone; polynomials whose ranges
-// overlap (offsets that are not monotone) are caught by the total the scan
-// kernel checks.
-__device__ __forceinline__ int checked_degree(const UnevenArgs &U, int64_t i, bool &consistent)
-{
-    int d = __ldg(U.degrees + i);
-    int64_t o0 = __ldg(U.offsets + i), o1 = __ldg(U.offsets + i + 1);
-    consistent = (o0 >= i) && (o1 >= o0) && (o1 <= U.n_coeffs - (U.n - 1 - i)) && (o1 - o0 == (int64_t)d + 1);
-    return (consistent && d >= 1 && d <= UNEVEN_MAX_DEG) ? d : -1;
-}
-
-// NaN roots of polynomial i (its offsets passed checked_degree's bounds).
-__device__ __forceinline__ void nan_roots(const UnevenArgs &U, int64_t i, double *roots)
-{
-    if (!roots) return;
-    const int dd = __ldg(U.degrees + i);
-    const int64_t r0 = __ldg(U.offsets + i) - i;
-    const double q = __longlong_as_double(0x7ff8000000000000ll);
-    for (int j = 0; j < dd; ++j) reinterpret_cast<double2 *>(roots)[r0 + j] = make_double2(q, q);
-}
-
 // Count polynomials per degree; mark the unsolvable ones DEGENERATE (NaN
 // roots where the offsets are consistent, nothing written where they are not).
 __global__ void __launch_bounds__(256) uneven_count_kernel(UnevenArgs U, UnevenHeader *hdr, double *roots,
@@ -256,7 +222,7 @@ size_t uneven_workspace_bytes(int64_t n, int64_t n_coeffs, rd_dtype dt)
 
 int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const int64_t *offsets, int64_t n,
                   int64_t n_coeffs, bool mixed, void *ws, const int *block, const int *cps, const int *lanes,
-                  const int *pw, bool fork, cudaStream_t st)
+                  const int *pw, bool fork, bool open_shape, cudaStream_t st)
 {
     UnevenLayout L = uneven_layout(ws, n);
     UnevenArgs U{degrees, offsets, n, n_coeffs};
@@ -269,6 +235,7 @@ int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const
     if (ctas < 1) ctas = 1;
     uneven_count_kernel<<<(unsigned)ctas, tb, 0, st>>>(U, L.hdr, a.roots, a.status, a.stats);
     if ((rc = rd_check_launch("uneven_count_kernel"))) return rc;
+    if (open_shape && uneven_group_takes(n, mixed)) return launch_uneven_group(a, dt, U, L.hdr, mixed, st);
     uneven_scan_kernel<<<1, 32, 0, st>>>(L.hdr, n_coeffs);
     if ((rc = rd_check_launch("uneven_scan_kernel"))) return rc;
     if (dt == RD_C64)

@@ -33,6 +33,39 @@ struct UnevenLayout {
     char *bins;
 };
 
+struct UnevenArgs {
+    const uint8_t *degrees;
+    const int64_t *offsets;
+    int64_t n;
+    int64_t n_coeffs;
+};
+
+// A polynomial is solvable when its offsets hold exactly degree + 1
+// coefficients, its degree is 1..12, and its roots fit the packed root array
+// of n_coeffs - n elements: o0 >= i keeps root 0 (at o0 - i) at or above 0,
+// o1 <= n_coeffs - (n - 1 - i) keeps its last root (at o1 - i - 2) below
+// n_coeffs - n. The comparisons are ordered so that no difference overflows.
+// These bounds hold for each polynomial alone; polynomials whose ranges
+// overlap (offsets that are not monotone) are caught by the total the scan
+// kernel checks.
+__device__ __forceinline__ int checked_degree(const UnevenArgs &U, int64_t i, bool &consistent)
+{
+    int d = __ldg(U.degrees + i);
+    int64_t o0 = __ldg(U.offsets + i), o1 = __ldg(U.offsets + i + 1);
+    consistent = (o0 >= i) && (o1 >= o0) && (o1 <= U.n_coeffs - (U.n - 1 - i)) && (o1 - o0 == (int64_t)d + 1);
+    return (consistent && d >= 1 && d <= UNEVEN_MAX_DEG) ? d : -1;
+}
+
+// NaN roots of polynomial i (its offsets passed checked_degree's bounds).
+__device__ __forceinline__ void nan_roots(const UnevenArgs &U, int64_t i, double *roots)
+{
+    if (!roots) return;
+    const int dd = __ldg(U.degrees + i);
+    const int64_t r0 = __ldg(U.offsets + i) - i;
+    const double q = __longlong_as_double(0x7ff8000000000000ll);
+    for (int j = 0; j < dd; ++j) reinterpret_cast<double2 *>(roots)[r0 + j] = make_double2(q, q);
+}
+
 // Largest batch the uneven path takes: n < 2^32 polynomials (32-bit slots)
 // and n_coeffs <= 2^40 coefficients, so that no workspace size wraps.
 constexpr int64_t UNEVEN_MAX_N = (int64_t)1 << 32;
@@ -64,6 +97,11 @@ inline UnevenLayout uneven_layout(void *ws, int64_t n)
 // they can be captured into a CUDA graph (as two parallel branches).
 int uneven_fork(cudaStream_t st, cudaStream_t *side, cudaEvent_t *fork, cudaEvent_t *join, bool retry = false);
 int uneven_join(cudaStream_t st, cudaStream_t side, cudaEvent_t join);
+
+// Small batches: every polynomial by a group of lanes, no bins (rd_group.cu).
+int launch_uneven_group(const SolveArgs &a, rd_dtype dt, const UnevenArgs &U, const UnevenHeader *hdr, bool mixed,
+                        cudaStream_t st);
+bool uneven_group_takes(int64_t n, bool mixed);
 
 // Solve every degree bin of a packed batch (one persistent kernel per
 // degree, largest degree first) with the per-degree launch shapes
