@@ -85,8 +85,8 @@ typedef struct {
                               only, degree 1 always runs one lane). Two lanes measured
                               slower on GB300 at degrees 6..12; the autotuner times both   */
     int32_t polish_warps;  /* RD_MIXED (either polish mode), one lane, rd_roots_batched and
-                              rd_roots_density: 0 = every warp sweeps and then polishes its
-                              own 32 polynomials; P > 0 = warp-specialised CTAs, P warps of
+                              rd_roots_density: 0 (with an explicit block or ctas_per_sm) =
+                              every warp sweeps and then polishes its own 32 polynomials; P > 0 = warp-specialised CTAs, P warps of
                               each polish, check, store and bin what the other block/32 - P
                               warps sweep, handed over through a shared-memory ring, so the
                               polish (FP64 pipe, or FP32 pipe with RD_POLISH_DF) and the

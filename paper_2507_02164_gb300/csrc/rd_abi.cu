@@ -138,6 +138,38 @@ bool shape_open(const rd_params &p)
     return p.block == 0 && p.ctas_per_sm == 0 && p.lanes == 0 && p.polish_warps == 0 && p.ring_slots == 0;
 }
 
+// The launch shape of a uniform batch too large for the small-batch solver,
+// when the caller left it open. Measured on complex-Gaussian polynomials (us,
+// 152 SMs; n = 120,000 / 200,000 / 2^20):
+//   FP64 polish, warp-specialised (512 threads with 9 polish warps up to degree
+//   6, 192 with 4 above) against one role with one warp per CTA: degree 4 79.6 /
+//   112 / 512 against 78.4 / 117 / 526, 5 114 / 175 / 806 against 115 / 175 / 814,
+//   6 153 / 236 / 1116 against 164 / 245 / 1193, 7 230 / 344 / 1570 against
+//   270 / 410 / 1895, 8 315 / 487 / 2193 against 348 / 535 / 2513; at 70,000 the
+//   ring's start and end cost more than the overlap gives (6: 103 against 101),
+//   from degree 9 the 255-register sweeps leave too few warps (9: 1658 against
+//   1596 for 2^19).
+//   Compensated polish, 256 threads against 32 (warps that start together
+//   share the instruction cache): degree 6 300,000 265 against 278, 2^20 904
+//   against 973; 8 571 against 616, 1959 against 2160; at 200,000 the last
+//   wave's coarser grain costs more (8: 420 against 403).
+//   Otherwise one warp per CTA, which spreads a ragged wave over all SMs: plain
+//   degree 6 65,536 1164 against 1285 with 128 threads, degree 12 20,000 2359
+//   against 3339; mixed degree 12 20,000 198 against 227; equal on full waves.
+void open_shape(rd_params &p, int degree, int64_t n, bool mixed)
+{
+    const int64_t per_sm = n / rd_sm_count_cached();
+    p.block = 32;
+    if (!mixed) return;
+    if (p.polish_mode == RD_POLISH_DF) {
+        if (degree >= 5 && per_sm >= 1536) p.block = 256;
+    } else if (degree >= 4 && degree <= 8 && per_sm >= (degree == 4 ? 1280 : 768)) {
+        const bool wide = degree == 5 || degree == 6;
+        p.block = wide ? 512 : 192;
+        p.polish_warps = wide ? 9 : 4;
+    }
+}
+
 // Validate a tile clip (host struct, device arrays) for n polynomials.
 int check_clip(const rd_clip &c, int64_t n)
 {
@@ -220,8 +252,10 @@ int solve_common(const void *coeffs, rd_dtype dtype, int degree, int64_t n, rd_m
     a.n = n;
     if (n == 0) return RD_OK;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if (shape_open(p) && rd::group_takes(degree, n, mode == RD_MIXED))
-        return rd::launch_group(degree, dtype, mode == RD_MIXED, a, st);
+    if (shape_open(p)) {
+        if (rd::group_takes(degree, n, mode == RD_MIXED)) return rd::launch_group(degree, dtype, mode == RD_MIXED, a, st);
+        open_shape(p, degree, n, mode == RD_MIXED);
+    }
     if (p.polish_warps > 0) {
         if (mode != RD_MIXED) return rd_set_error(RD_EINVAL, "params.polish_warps > 0 needs RD_MIXED");
         return rd::launch_solve_ws(degree, dtype, a, p.block, p.ctas_per_sm, p.polish_warps, p.ring_slots, st);
