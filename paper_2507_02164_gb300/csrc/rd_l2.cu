@@ -21,7 +21,9 @@
 //   * double-float sums (l2_kernel_df): lane q owns angle theta_q; radial sums
 //     u_j(q) = sum_p (w_p r_p^{j+1}) g_pq, then v_j = sum_q u_j(q) e^{-i j theta_q}
 //     by a warp reduce-scatter.
+#include <atomic>
 #include <cmath>
+#include <mutex>
 
 #include "rd_common.cuh"
 
@@ -331,71 +333,75 @@ __global__ void __launch_bounds__(256, 2) l2_kernel_df(const double2 *__restrict
     }
 }
 
-int launch_l2(const double *samples, int64_t n, int nr, int degree, double *coeffs, int precision,
-              cudaStream_t st)
+// The tables of a node count, built on its first use and kept (host memory,
+// 24 KB per node count, at most 32 of them): building them takes 80 us at nr
+// = 16 and 200 us at 24 (nodes by Newton's method, powers), more than the
+// kernel takes on a few thousand sub-disks. They hold every coefficient up to
+// L2_MAX_DEG; the kernels read those of their degree.
+struct L2HostTables {
+    L2Tables fp64;
+    L2TablesDF df;
+};
+
+static const L2HostTables &l2_tables(int nr)
 {
-    if (precision == 1) {
-        L2TablesDF T;
+    static L2HostTables tables[L2_MAX_NR + 1];
+    static std::atomic<bool> ready[L2_MAX_NR + 1];
+    static std::mutex mu;
+    L2HostTables *t = &tables[nr];
+    if (ready[nr].load(std::memory_order_acquire)) return *t;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!ready[nr].load(std::memory_order_relaxed)) {
         double r[L2_MAX_NR], w[L2_MAX_NR];
         l2_nodes_host(nr, r, w);
         const double pi = 3.14159265358979323846;
-        for (int p = 0; p < L2_MAX_NR; ++p)
+        for (int p = 0; p < nr; ++p)
             for (int j = 0; j <= L2_MAX_DEG; ++j) {
-                double v = 0.0;
-                if (p < nr && j <= degree) v = w[p] * std::pow(r[p], j + 1) * (2.0 * pi / L2_NT) * (j + 1) / pi;
+                const double v = w[p] * std::pow(r[p], j + 1) * (2.0 * pi / L2_NT) * (j + 1) / pi;
                 const float h = (float)v, l = (float)(v - (double)h);
-                T.whi[p][j] = make_float2(h, h);
-                T.wlo[p][j] = make_float2(l, l);
+                t->fp64.wr[p][j] = v;
+                t->df.whi[p][j] = make_float2(h, h);
+                t->df.wlo[p][j] = make_float2(l, l);
             }
         for (int j = 0; j <= L2_MAX_DEG; ++j)
             for (int q = 0; q < L2_NT; ++q) {
-                int t = (j * q) % L2_NT;
-                double ang = 2.0 * pi * t / L2_NT;
-                double c = std::cos(ang), sn = -std::sin(ang);
-                T.thi[j][q][0] = (float)c;
-                T.tlo[j][q][0] = (float)(c - (double)T.thi[j][q][0]);
-                T.thi[j][q][1] = (float)sn;
-                T.tlo[j][q][1] = (float)(sn - (double)T.thi[j][q][1]);
+                // e^{-i j theta_q}, theta_q = 2 pi q / nt, reduced exactly: (j q) mod nt
+                const double ang = 2.0 * pi * ((j * q) % L2_NT) / L2_NT;
+                const double c[2] = {std::cos(ang), -std::sin(ang)};
+                for (int k = 0; k < 2; ++k) {
+                    t->fp64.tw[j][q][k] = c[k];
+                    t->df.thi[j][q][k] = (float)c[k];
+                    t->df.tlo[j][q][k] = (float)(c[k] - (double)t->df.thi[j][q][k]);
+                }
             }
+        ready[nr].store(true, std::memory_order_release);
+    }
+    return *t;
+}
+
+int launch_l2(const double *samples, int64_t n, int nr, int degree, double *coeffs, int precision,
+              cudaStream_t st)
+{
+    const double2 *sp = reinterpret_cast<const double2 *>(samples);
+    double2 *cp = reinterpret_cast<double2 *>(coeffs);
+    const int64_t sms = rd_sm_count_cached();
+    if (precision == 1) {
+        const L2TablesDF &T = l2_tables(nr).df;
         const int block = 256;
         int64_t ctas = (n + 7) / 8;
-        int64_t cap = (int64_t)rd_sm_count_cached() * 8;
-        if (ctas > cap) ctas = cap;
-        if (ctas < 1) ctas = 1;
-        const double2 *sp = reinterpret_cast<const double2 *>(samples);
-        double2 *cp = reinterpret_cast<double2 *>(coeffs);
+        if (ctas > sms * 8) ctas = sms * 8;
         if (nr == 16 && degree == 6)  // the full pipeline's 16 x 32 nodes and degree-6 fits
             l2_kernel_df<16, 6><<<(unsigned)ctas, block, 0, st>>>(sp, n, nr, degree, cp, T);
         else
             l2_kernel_df<0, -1><<<(unsigned)ctas, block, 0, st>>>(sp, n, nr, degree, cp, T);
         return rd_check_launch("l2_kernel_df");
     }
-    L2Tables T;
-    double r[L2_MAX_NR], w[L2_MAX_NR];
-    l2_nodes_host(nr, r, w);
-    const double pi = 3.14159265358979323846;
-    for (int p = 0; p < L2_MAX_NR; ++p)
-        for (int j = 0; j <= L2_MAX_DEG; ++j) {
-            double v = 0.0;
-            if (p < nr && j <= degree) v = w[p] * std::pow(r[p], j + 1) * (2.0 * pi / L2_NT) * (j + 1) / pi;
-            T.wr[p][j] = v;
-        }
-    for (int j = 0; j <= L2_MAX_DEG; ++j)
-        for (int q = 0; q < L2_NT; ++q) {
-            // e^{-i j theta_q}, theta_q = 2 pi q / nt, reduced exactly: (j q) mod nt
-            int t = (j * q) % L2_NT;
-            double ang = 2.0 * pi * t / L2_NT;
-            T.tw[j][q][0] = std::cos(ang);
-            T.tw[j][q][1] = -std::sin(ang);
-        }
+    const L2Tables &T = l2_tables(nr).fp64;
     // 8 warps per CTA; fewer while a small n would leave SMs without a CTA
-    const int64_t sms = rd_sm_count_cached();
     const int64_t warps = n >= sms * L2_WARPS ? L2_WARPS : (n + sms - 1) / sms;
     const int block = 32 * (int)warps;
     int64_t ctas = (n + warps - 1) / warps;
     if (ctas > sms * 8) ctas = sms * 8;
-    const double2 *sp = reinterpret_cast<const double2 *>(samples);
-    double2 *cp = reinterpret_cast<double2 *>(coeffs);
     if (nr == 16 && degree == 6)
         l2_kernel<16, 6><<<(unsigned)ctas, block, 0, st>>>(sp, n, nr, degree, cp, T);
     else
