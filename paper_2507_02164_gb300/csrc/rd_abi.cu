@@ -151,8 +151,9 @@ bool shape_open(const rd_params &p)
 //   1596 for 2^19).
 //   Compensated polish, 256 threads against 32 (warps that start together
 //   share the instruction cache): degree 6 300,000 265 against 278, 2^20 904
-//   against 973; 8 571 against 616, 1959 against 2160; at 200,000 the last
-//   wave's coarser grain costs more (8: 420 against 403).
+//   against 973; 9 740 against 784; at 200,000 the last wave's coarser grain
+//   costs more (10: 677 against 649). Degrees 7 and 8, at 168 registers: 128
+//   threads, three CTAs per SM (8 2^19 1019 against 1105 with 256).
 //   Otherwise one warp per CTA, which spreads a ragged wave over all SMs: plain
 //   degree 6 65,536 1164 against 1285 with 128 threads, degree 12 20,000 2359
 //   against 3339; mixed degree 12 20,000 198 against 227; equal on full waves.
@@ -162,7 +163,8 @@ void open_shape(rd_params &p, int degree, int64_t n, bool mixed)
     p.block = 32;
     if (!mixed) return;
     if (p.polish_mode == RD_POLISH_DF) {
-        if (degree >= 5 && per_sm >= 1536) p.block = 256;
+        if (degree == 7 || degree == 8) p.block = 128;
+        else if (degree >= 5 && per_sm >= 1536) p.block = 256;
     } else if (degree >= 4 && degree <= 8 && per_sm >= (degree == 4 ? 1280 : 768)) {
         const bool wide = degree == 5 || degree == 6;
         p.block = wide ? 512 : 192;

@@ -758,9 +758,18 @@ __device__ __forceinline__ void solve_warp(const SolveArgs &A, const void *coeff
     finish_lane<N, T, In, MODE>(A, coeffs, n, i, map, S, d, degenerate, not_conv);
 }
 
+// Degrees 7 and 8 with FP32 sweeps fit 168 registers without spilling (left
+// alone the compiler takes 172 to 201, which costs one to two of the twelve
+// warps per SM that 168 allow). Measured (us, 168 against 172-201 registers at
+// the best block of each): FP64 polish degree 7 2^19 874 against 974, 8 1184
+// against 1286, 100,003 254 against 272; compensated polish 7 718 against 769,
+// 8 100,003 190 against 212. Degree 9 spills 316 B and gains nothing (1615
+// against 1595), 10 and up lose (1084 against 1017).
+__host__ __device__ constexpr bool solve_twelve_warps(int n, int mode) { return mode != MODE_PLAIN && (n == 7 || n == 8); }
+
 // Uniform batch: warps stride over A.n polynomials, 32 at a time.
 template <int N, typename T, typename In, int MODE>
-__global__ void __launch_bounds__(256, (MODE != MODE_PLAIN && N <= 6) ? 2 : 1) solve_kernel(SolveArgs A)
+__device__ __forceinline__ void solve_uniform(const SolveArgs &A)
 {
     const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int64_t warp_id = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -770,6 +779,18 @@ __global__ void __launch_bounds__(256, (MODE != MODE_PLAIN && N <= 6) ? 2 : 1) s
     for (int64_t base = warp_id * 32; base < A.n; base += warps_total * 32)
         solve_warp<N, T, In, MODE>(A, A.coeffs, A.n, base, map, S);
     stats_end(S, A.stats);
+}
+
+template <int N, typename T, typename In, int MODE>
+__global__ void __launch_bounds__(256, (MODE != MODE_PLAIN && N <= 6) ? 2 : 1) solve_kernel(SolveArgs A)
+{
+    solve_uniform<N, T, In, MODE>(A);
+}
+
+template <int N, typename T, typename In, int MODE>
+__global__ void __maxnreg__(168) solve_kernel_r168(SolveArgs A)
+{
+    solve_uniform<N, T, In, MODE>(A);
 }
 
 }  // namespace rd

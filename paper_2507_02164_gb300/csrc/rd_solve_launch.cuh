@@ -6,11 +6,20 @@
 
 namespace rd {
 
+template <int N, typename T, typename In, int MODE>
+static auto solve_kernel_of()
+{
+    if constexpr (solve_twelve_warps(N, MODE))
+        return solve_kernel_r168<N, T, In, MODE>;
+    else
+        return solve_kernel<N, T, In, MODE>;
+}
+
 template <int N, typename In, int MODE>
 static int launch_one(const SolveArgs &a, int block, int ctas_per_sm, cudaStream_t st)
 {
     using T = typename std::conditional<MODE != MODE_PLAIN, float, double>::type;
-    auto kern = solve_kernel<N, T, In, MODE>;
+    auto kern = solve_kernel_of<N, T, In, MODE>();
     int per_sm = ctas_per_sm;
     if (per_sm <= 0) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, 0) != cudaSuccess || per_sm < 1)
