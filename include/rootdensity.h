@@ -279,10 +279,12 @@ int rd_pointer_is_device_accessible(const void *p);
  * before and after it. The first call on a device from a host thread creates
  * the helper stream and its two events; make that call outside capture.
  * (With the launch shape open -- no tuning, no shape in params -- a small batch
- * is solved without bins, in 3 launches on `stream` and no helper stream.) */
+ * is solved without bins, in 3 launches on `stream` and no helper stream; a
+ * degree whose tuning entries are all 0 keeps its shape open.) */
 typedef struct {
     /* Launch shape of each degree bin's solve kernel, indexed by the degree
-     * (entries 1..12; entries 0 and 13..15 are ignored). 0 = the default.   */
+     * (entries 1..12; entries 0 and 13..15 are ignored). 0 = the default; with
+     * all four 0 (and no shape in params) the library picks the form too.   */
     int32_t block[16];        /* threads per CTA, a multiple of 32 in [32, 256]                  */
     int32_t ctas_per_sm[16];  /* resident CTAs per SM (0 = the occupancy maximum)                 */
     int32_t lanes[16];        /* lanes per polynomial, 1 or 2 (0 = params.lanes)                  */

@@ -30,9 +30,10 @@ int l2_nodes_host(int nr, double *r, double *w);
 size_t uneven_workspace_bytes(int64_t n, int64_t n_coeffs, rd_dtype dt);
 int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const int64_t *offsets, int64_t n,
                   int64_t n_coeffs, bool mixed, void *ws, const int *block, const int *cps, const int *lanes,
-                  const int *pw, bool fork, bool open_shape, cudaStream_t st);
+                  const int *pw, bool fork, const bool *open_shape, cudaStream_t st);
 bool group_takes(int degree, int64_t n, bool mixed);
 int launch_group(int degree, rd_dtype dt, bool mixed, const SolveArgs &a, cudaStream_t st);
+int launch_solve_split(int degree, rd_dtype dt, const SolveArgs &a, cudaStream_t st);
 int launch_l2(const double *samples, int64_t n, int nr, int degree, double *coeffs, int precision,
               cudaStream_t st);
 int roots_uneven_common(const void *coeffs, rd_dtype dtype, const uint8_t *degrees, const int64_t *offsets, int64_t n,
@@ -138,37 +139,44 @@ bool shape_open(const rd_params &p)
     return p.block == 0 && p.ctas_per_sm == 0 && p.lanes == 0 && p.polish_warps == 0 && p.ring_slots == 0;
 }
 
-// The launch shape of a uniform batch too large for the small-batch solver,
-// when the caller left it open. Measured on complex-Gaussian polynomials (us,
-// 152 SMs; n = 120,000 / 200,000 / 2^20):
-//   FP64 polish, warp-specialised (512 threads with 9 polish warps up to degree
-//   6, 192 with 4 above) against one role with one warp per CTA: degree 4 79.6 /
-//   112 / 512 against 78.4 / 117 / 526, 5 114 / 175 / 806 against 115 / 175 / 814,
-//   6 153 / 236 / 1116 against 164 / 245 / 1193, 7 230 / 344 / 1570 against
-//   270 / 410 / 1895, 8 315 / 487 / 2193 against 348 / 535 / 2513; at 70,000 the
-//   ring's start and end cost more than the overlap gives (6: 103 against 101),
-//   from degree 9 the 255-register sweeps leave too few warps (9: 1658 against
-//   1596 for 2^19).
-//   Compensated polish, 256 threads against 32 (warps that start together
-//   share the instruction cache): degree 6 300,000 265 against 278, 2^20 904
-//   against 973; 9 740 against 784; at 200,000 the last wave's coarser grain
-//   costs more (10: 677 against 649). Degrees 7 and 8, at 168 registers: 128
-//   threads, three CTAs per SM (8 2^19 1019 against 1105 with 256).
-//   Otherwise one warp per CTA, which spreads a ragged wave over all SMs: plain
-//   degree 6 65,536 1164 against 1285 with 128 threads, degree 12 20,000 2359
-//   against 3339; mixed degree 12 20,000 198 against 227; equal on full waves.
+// The FP64 polish of a large enough batch takes the split-register
+// warp-specialised solver (rd_solve_split.cuh). Measured on complex-Gaussian
+// polynomials (us, 152 SMs), split against the best other form:
+//   degree     n 40,000     60,000     80,000    100,003    150,000    2^19
+//    4            41 / 33    48 / 43    62 / 58    66 / 68    86 / 88    251 / 266 (complex128 315 / 310)
+//    5            58 / 49    75 / 66    82 / 84    97 / 103  127 / 133   379 / 407
+//    6            76 / 69    96 / 91   123 / 116  133 / 139  178 / 186   527 / 571
+//    7           103 / 89   131 / 141  146 / 164  178 / 191  234 / 267   716 / 828
+//    8           131 / 120  164 / 188  189 / 227  227 / 261  305 / 366   973 / 1141
+//    9           180 / 200  193 / 222  270 / 318  285 / 340  389 / 470  1253 / 1598
+//   10           220 / 256  234 / 276  328 / 399  344 / 423  470 / 584  1506 / 1996
+//   12           342 / 410  409 / 453  562 / 644  626 / 707  874 / 983  2811 / 3229
+// (25,000: 9 116 / 112, 12 234 / 211). 2^24 Littlewood polynomials: 15.9 against
+// 17.3 ms.
+bool split_takes(int degree, rd_dtype dtype, int64_t n, bool mixed, int polish_mode)
+{
+    if (!mixed || polish_mode != RD_POLISH_FP64 || degree < 4) return false;
+    const int64_t per_sm = n / rd_sm_count_cached();
+    if (degree == 4) return dtype == RD_C64 && per_sm >= 640;
+    return per_sm >= (degree <= 6 ? 576 : (degree <= 8 ? 352 : 224));
+}
+
+// The launch shape of any other uniform batch too large for the small-batch
+// solver, when the caller left it open. Compensated polish: 256 threads against
+// 32 (warps that start together share the instruction cache) degree 6 300,000
+// 265 against 278 us, 2^20 904 against 973; 9 740 against 784; at 200,000 the last
+// wave's coarser grain costs more (10: 677 against 649); degrees 7 and 8, at 168
+// registers: 128 threads, three CTAs per SM (8 2^19 1019 against 1105 with
+// 256). Otherwise one warp per CTA, which spreads a ragged wave over all SMs:
+// plain degree 6 65,536 1164 against 1285 with 128 threads, degree 12 20,000 2359
+// against 3339; mixed degree 12 20,000 198 against 227; equal on full waves.
 void open_shape(rd_params &p, int degree, int64_t n, bool mixed)
 {
     const int64_t per_sm = n / rd_sm_count_cached();
     p.block = 32;
-    if (!mixed) return;
-    if (p.polish_mode == RD_POLISH_DF) {
+    if (mixed && p.polish_mode == RD_POLISH_DF) {
         if (degree == 7 || degree == 8) p.block = 128;
         else if (degree >= 5 && per_sm >= 1536) p.block = 256;
-    } else if (degree >= 4 && degree <= 8 && per_sm >= (degree == 4 ? 1280 : 768)) {
-        const bool wide = degree == 5 || degree == 6;
-        p.block = wide ? 512 : 192;
-        p.polish_warps = wide ? 9 : 4;
     }
 }
 
@@ -256,6 +264,7 @@ int solve_common(const void *coeffs, rd_dtype dtype, int degree, int64_t n, rd_m
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (shape_open(p)) {
         if (rd::group_takes(degree, n, mode == RD_MIXED)) return rd::launch_group(degree, dtype, mode == RD_MIXED, a, st);
+        if (split_takes(degree, dtype, n, mode == RD_MIXED, p.polish_mode)) return rd::launch_solve_split(degree, dtype, a, st);
         open_shape(p, degree, n, mode == RD_MIXED);
     }
     if (p.polish_warps > 0) {
@@ -440,7 +449,10 @@ int roots_uneven_common(const void *coeffs, rd_dtype dtype, const uint8_t *degre
     size_t need = rd::uneven_workspace_bytes(n, n_coeffs, dtype);
     if (ws_bytes < need) return rd_set_error(RD_EINVAL, "workspace too small: %zu < %zu bytes", ws_bytes, need);
     int block[16], cps[16], lanes[16], pw[16];
+    bool open[16];  // this degree's launch shape is the library's choice
     for (int d = 0; d < 16; ++d) {
+        open[d] = shape_open(p) && !(tuning && d >= 1 && d <= 12 &&
+                                     (tuning->block[d] || tuning->ctas_per_sm[d] || tuning->lanes[d] || tuning->polish_warps[d]));
         block[d] = p.block ? p.block : 128;
         cps[d] = p.ctas_per_sm;
         lanes[d] = p.lanes;
@@ -479,7 +491,7 @@ int roots_uneven_common(const void *coeffs, rd_dtype dtype, const uint8_t *degre
     a.coeffs = coeffs;
     a.n = n;
     return rd::launch_uneven(a, dtype, degrees, offsets, n, n_coeffs, mode == RD_MIXED, ws, block, cps, lanes, pw,
-                             fork, !tuning && shape_open(p), reinterpret_cast<cudaStream_t>(stream));
+                             fork, open, reinterpret_cast<cudaStream_t>(stream));
 }
 
 }  // namespace rd

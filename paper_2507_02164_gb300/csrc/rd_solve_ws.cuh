@@ -133,6 +133,18 @@ __device__ __forceinline__ bool ws_put(WsCtl *ctl, WsSlot<N> *ring, int slots, u
     return true;
 }
 
+// A task that its polish warp could not take: polynomial i is reported, not solved.
+template <class Map>
+__device__ __forceinline__ void ws_report_abandoned(const SolveArgs &A, const Map &map, const CtaStats &S, int64_t i,
+                                                    int64_t n)
+{
+    const bool valid = i < n;
+    if (valid && A.status) A.status[map.poly(i)] = RD_STATUS_REJECTED;
+    S.add(ST_POLYS, valid ? 1u : 0u);
+    S.add(ST_STATUS0 + RD_STATUS_REJECTED, valid ? 1u : 0u);
+    S.add(ST_TIMEOUT, valid ? 1u : 0u);
+}
+
 // The polish role of a warp-specialised CTA: take polish tickets until the
 // CTA's my_tasks tasks are done; each task's slot is emptied and its 32
 // polynomials finished (finish_lane). A task whose slot never fills (the CTA
@@ -152,12 +164,7 @@ __device__ __forceinline__ void ws_polish_role(const SolveArgs &A, const void *c
         const int64_t i = (b + (int64_t)k * G) * 32 + lane;
         const unsigned slot = k % (unsigned)slots, round = k / (unsigned)slots;
         if (!ws_wait(&ctl->state[slot], 2u * round + 1u, abort_flag)) {
-            // abandoned: its polynomials are reported, not solved
-            const bool valid = i < n;
-            if (valid && A.status) A.status[map.poly(i)] = RD_STATUS_REJECTED;
-            S.add(ST_POLYS, valid ? 1u : 0u);
-            S.add(ST_STATUS0 + RD_STATUS_REJECTED, valid ? 1u : 0u);
-            S.add(ST_TIMEOUT, valid ? 1u : 0u);
+            ws_report_abandoned(A, map, S, i, n);
             continue;
         }
         const WsSlot<N> &w = ring[slot];

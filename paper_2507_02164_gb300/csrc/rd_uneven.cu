@@ -220,9 +220,21 @@ size_t uneven_workspace_bytes(int64_t n, int64_t n_coeffs, rd_dtype dt)
     return uneven_bytes(n, n_coeffs, dt == RD_C64 ? 8 : 16);
 }
 
+// Whether the degree bins 4 to 12 take the split-register solver
+// (rd_solve_split.cuh) where the caller left their launch shapes open. The
+// bins' sizes exist only on the device, so the line is drawn on n; each split
+// kernel takes whole SMs, so small bins lose the overlap of the two chains.
+// Measured (us, degrees 2..12, complex64, split / one role): 300,000 1030 / 930,
+// 2^19 1560 / 1430, 2^20 2385 / 2498, 2^22 7909 / 9357 (complex128 2574 / 2621,
+// 8702 / 9864).
+static bool uneven_split_takes(int64_t n, bool mixed, int polish_mode)
+{
+    return mixed && polish_mode == RD_POLISH_FP64 && n >= (int64_t)6144 * rd_sm_count_cached();
+}
+
 int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const int64_t *offsets, int64_t n,
                   int64_t n_coeffs, bool mixed, void *ws, const int *block, const int *cps, const int *lanes,
-                  const int *pw, bool fork, bool open_shape, cudaStream_t st)
+                  const int *pw, bool fork, const bool *open_shape, cudaStream_t st)
 {
     UnevenLayout L = uneven_layout(ws, n);
     UnevenArgs U{degrees, offsets, n, n_coeffs};
@@ -235,7 +247,13 @@ int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const
     if (ctas < 1) ctas = 1;
     uneven_count_kernel<<<(unsigned)ctas, tb, 0, st>>>(U, L.hdr, a.roots, a.status, a.stats);
     if ((rc = rd_check_launch("uneven_count_kernel"))) return rc;
-    if (open_shape && uneven_group_takes(n, mixed)) return launch_uneven_group(a, dt, U, L.hdr, mixed, st);
+    bool all_open = true;
+    for (int d = 1; d <= UNEVEN_MAX_DEG; ++d) all_open &= open_shape[d];
+    if (all_open && uneven_group_takes(n, mixed)) return launch_uneven_group(a, dt, U, L.hdr, mixed, st);
+    int bins_pw[16];
+    const bool split = uneven_split_takes(n, mixed, a.polish_mode);
+    for (int d = 0; d < 16; ++d) bins_pw[d] = split && open_shape[d] && d >= 4 && d <= UNEVEN_MAX_DEG ? UNEVEN_SPLIT : pw[d];
+    pw = bins_pw;
     uneven_scan_kernel<<<1, 32, 0, st>>>(L.hdr, n_coeffs);
     if ((rc = rd_check_launch("uneven_scan_kernel"))) return rc;
     if (dt == RD_C64)

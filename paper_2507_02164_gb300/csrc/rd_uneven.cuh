@@ -98,6 +98,11 @@ inline UnevenLayout uneven_layout(void *ws, int64_t n)
 int uneven_fork(cudaStream_t st, cudaStream_t *side, cudaEvent_t *fork, cudaEvent_t *join, bool retry = false);
 int uneven_join(cudaStream_t st, cudaStream_t side, cudaEvent_t join);
 
+// Large bins, FP64 polish: the split-register solver (rd_solve_split.cuh).
+int launch_uneven_split(int degree, rd_dtype dt, const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets,
+                        cudaStream_t st);
+constexpr int UNEVEN_SPLIT = -1;  // in launch_uneven_bins' pw[d]
+
 // Small batches: every polynomial by a group of lanes, no bins (rd_group.cu).
 int launch_uneven_group(const SolveArgs &a, rd_dtype dt, const UnevenArgs &U, const UnevenHeader *hdr, bool mixed,
                         cudaStream_t st);
@@ -106,7 +111,8 @@ bool uneven_group_takes(int64_t n, bool mixed);
 // Solve every degree bin of a packed batch (one persistent kernel per
 // degree, largest degree first) with the per-degree launch shapes
 // block[d], cps[d], lanes per polynomial lanes[d] and polish warps pw[d]
-// (> 0: the warp-specialised form, mixed mode, degrees up to 8).
+// (> 0: the warp-specialised form, mixed mode, degrees up to 8; UNEVEN_SPLIT:
+// the split-register form, FP64 polish, degrees 4 to 12).
 template <typename In, int MODE>
 int launch_uneven_bins(const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets, const int *block,
                        const int *cps, const int *lanes, const int *pw, bool fork, cudaStream_t st);

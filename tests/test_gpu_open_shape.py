@@ -36,8 +36,8 @@ def _same(a, b):
     assert a[3]["wait_timeouts"] == 0
 
 
-@pytest.mark.parametrize("degree,per_sm,polish", [(4, 1280, "fp64"), (5, 768, "fp64"), (6, 768, "fp64"), (7, 768, "fp64"),
-                                                  (8, 768, "fp64"), (9, 768, "fp64"), (4, 1536, "df"), (5, 1536, "df"),
+@pytest.mark.parametrize("degree,per_sm,polish", [(4, 640, "fp64"), (6, 576, "fp64"), (8, 352, "fp64"),
+                                                  (9, 224, "fp64"), (7, 1536, "df"), (5, 1536, "df"),
                                                   (8, 1536, "df")])
 def test_open_shape_is_one_role_bit_for_bit(dev, degree, per_sm, polish):
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
