@@ -92,7 +92,7 @@ __device__ __forceinline__ void finish_lean(const SolveArgs &A, const void *coef
     const int lane = threadIdx.x & 31;
     const bool valid = i < n;
     uint8_t st = degenerate ? RD_STATUS_DEGENERATE : (not_conv ? RD_STATUS_NOT_CONVERGED : RD_STATUS_OK);
-    unsigned newton = 0;
+    unsigned newton = 0, extra = 0;  // extra: steps taken for any of the warp's polynomials
     const bool polish = A.polish_steps > 0 || A.polish_extra > 0;
     auto ad = [&](int k) -> cx<double> {
         const double2 v = mem.ad[k][lane];
@@ -193,25 +193,59 @@ __device__ __forceinline__ void finish_lean(const SolveArgs &A, const void *coef
         }
         if (degenerate) failed = 0;
         if (A.polish_extra > 0 && __any_sync(0xffffffffu, failed != 0)) {
+            // Further steps with p and p' both in FP64. The failed roots of the
+            // whole warp go to one lane each, whichever polynomial they belong to
+            // (everything they need is in shared memory): a warp whose polynomials
+            // fail on all roots takes one pass instead of N (129,600 sub-disks of
+            // the full pipeline, some 100 of whose 4,050 warps have rejected
+            // polynomials: 484 -> 470 us). The slot's eigenvalues are no longer
+            // needed; it holds the list (lane, root).
+            unsigned *list = reinterpret_cast<unsigned *>(&slot.d[0][0]);
+            unsigned at = __popc(failed);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned v = __shfl_up_sync(0xffffffffu, at, o);
+                at += lane >= o ? v : 0u;
+            }
+            const unsigned total = __shfl_sync(0xffffffffu, at, 31);
+            const unsigned begin = at - __popc(failed);
+            __syncwarp();
+            at = begin;
+            for (unsigned m = failed; m; m &= m - 1u) list[at++] = (unsigned)lane | ((unsigned)(__ffs(m) - 1) << 8);
+            __syncwarp();
 #pragma unroll 1
-            for (int j = 0; j < N; ++j) {
-                if (!((failed >> j) & 1u)) continue;
-                cx<double> zj = root(j);
-                for (int it = 0; ((failed >> j) & 1u) && it < A.polish_extra; ++it) {
-                    cx<double> p = ad(N), dp = {0.0, 0.0};
+            for (unsigned t = lane; t < total; t += 32) {
+                const int l = (int)(list[t] & 31u), j = (int)(list[t] >> 8);
+                auto adl = [&](int k) -> cx<double> { return {mem.ad[k][l].x, mem.ad[k][l].y}; };
+                cx<double> zj = {mem.z[j][l].x, mem.z[j][l].y};
+                bool good = false;
+                for (int it = 0; !good && it < A.polish_extra; ++it) {
+                    cx<double> p = adl(N), dp = {0.0, 0.0};
 #pragma unroll 1
                     for (int k = N - 1; k >= 0; --k) {
                         dp = cfma(dp, zj, p);
-                        p = cfma(p, zj, ad(k));
+                        p = cfma(p, zj, adl(k));
                     }
                     const cx<double> dz = cdiv(p, dp);
                     if (!(finite_bits(dz.re) && finite_bits(dz.im))) break;
                     zj = sub(zj, dz);
-                    newton += 1;
-                    if (passes(horner(zj), zj)) failed &= ~(1u << j);
+                    extra += 1;
+                    cx<double> q = adl(N);
+                    const float az = sqrtf(norm2(d2f(zj)));
+                    float den = abs1(cx<float>{mem.af[N][l].x, mem.af[N][l].y});
+#pragma unroll 1
+                    for (int k = N - 1; k >= 0; --k) {
+                        q = cfma(q, zj, adl(k));
+                        den = fmaf(den, az, abs1(cx<float>{mem.af[k][l].x, mem.af[k][l].y}));
+                    }
+                    good = (sqrtf(norm2(d2f(q))) <= rtol * den) && finite_bits(zj.re) && finite_bits(zj.im);
                 }
-                mem.z[j][lane] = make_double2(zj.re, zj.im);
+                mem.z[j][l] = make_double2(zj.re, zj.im);
+                list[t] = good ? 1u : 0u;
             }
+            __syncwarp();
+            at = begin;
+            for (unsigned m = failed; m; m &= m - 1u) failed &= ~(list[at++] << (__ffs(m) - 1));
             __syncwarp();
         }
         bool reject = failed != 0;
@@ -243,7 +277,7 @@ __device__ __forceinline__ void finish_lean(const SolveArgs &A, const void *coef
         }
         if (reject && st == RD_STATUS_OK && !degenerate) st = RD_STATUS_REJECTED;
     }
-    const unsigned nw = degenerate ? 0u : newton, nr = (degenerate || !polish) ? 0u : (unsigned)N;
+    const unsigned nw = (degenerate ? 0u : newton) + extra, nr = (degenerate || !polish) ? 0u : (unsigned)N;
     S.add(ST_NEWTON, nw);
     S.add(ST_F64, (8u * N + 2u) * nw + (8u * N + 4u) * nr);
     S.add(ST_F32, (8u * N + 3u) * nw + (2u * N + 4u) * nr);
