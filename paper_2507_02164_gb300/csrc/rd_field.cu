@@ -13,13 +13,13 @@
 // array of 16 x 32 samples per sub-disk (1.06 GB for the 480 x 270 tiles)
 // that the caller must have made. Here nothing but the histogram (and, if
 // asked, coefficients, roots and status) touches memory:
-//   * one warp takes 32 consecutive tiles; for each tile, lane q evaluates f
+//   * one warp takes up to 32 consecutive tiles; for each tile, lane q evaluates f
 //     in FP64 at the 16 nodes r_p e^{i theta_q} of its angle and stages them
 //     in shared memory; the radial sums are double-float sums on the FP32
 //     pipe (the samples scaled by the tile's largest power of two, as in
 //     l2_kernel_df), the angular sums a warp reduce-scatter; the 7
 //     coefficients of the tile go to shared memory;
-//   * after 32 tiles the same warp solves them, one lane per tile
+//   * then the same warp solves them, one lane per tile
 //     (solve_warp: FP32 sweeps + FP64 polish, or FP64 sweeps), maps each root
 //     to z = c + rho w, keeps it when it lies in the tile's own cell of the
 //     grid and bins it.
@@ -47,6 +47,7 @@ struct FieldArgs {
     double poly[FIELD_MAX_POLY + 1][2];
     double xmin, ymax, tw, th;  // tile grid: top-left corner, tile width and height
     int nx, ny;
+    int group;                               // tiles a warp fits before it solves them, 1 .. 32
     double rho;                              // sub-disk radius
     double r[FIELD_NR];                      // Gauss-Legendre radii on [0, 1]
     double ct[FIELD_NT], st[FIELD_NT];       // cos, sin theta_q, theta_q = 2 pi q / 32
@@ -135,12 +136,14 @@ __global__ void __launch_bounds__(FIELD_WARPS * 32, MODE != MODE_PLAIN ? 2 : 1)
     }
     const CtaStats S = stats_begin(acc, A.stats);  // its barrier (when stats are kept) publishes s_tw
     if (!A.stats) __syncthreads();
+    // Groups go to warp 0 of every CTA, then to warp 1 of every CTA, ...: the
+    // last round, rarely full, is spread over all SMs.
     const int64_t ntiles = (int64_t)F.nx * F.ny;
-    const int64_t groups = (ntiles + 31) / 32;
+    const int64_t groups = (ntiles + F.group - 1) / F.group;
     const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + wid; g < groups; g += warps_total) {
-        const int64_t base = g * 32;
-        const int count = (int)(ntiles - base < 32 ? ntiles - base : 32);
+    for (int64_t g = (int64_t)wid * gridDim.x + blockIdx.x; g < groups; g += warps_total) {
+        const int64_t base = g * F.group;
+        const int count = (int)(ntiles - base < F.group ? ntiles - base : F.group);
 #pragma unroll 1
         for (int t = 0; t < count; ++t) {
             const int64_t tile = base + t;
@@ -312,11 +315,18 @@ static int launch_field_n(const SolveArgs &a, const rd_field_spec &spec, int fun
             per_sm < 1)
             per_sm = 1;
     }
-    const int64_t groups = ((int64_t)spec.nx * spec.ny + 31) / 32;
+    // Tiles per group: a warp's share of the tiles in equal rounds of at most 32
+    // (480 x 270 over 2,432 warps: two rounds of 27, where rounds of 32 left the
+    // second one two thirds full and on a third of the SMs), and 1 while there are
+    // fewer tiles than warps: fitting a tile takes 976 FP64 instructions, solving a
+    // group about 500 whatever its size. Measured: 480 x 270 9.25 -> 7.94 ms, 200 x
+    // 112 2.80 -> 1.61 ms, 40 x 22 2,570 -> 202 us.
+    const int64_t ntiles = (int64_t)spec.nx * spec.ny;
     int64_t grid = (int64_t)per_sm * rd_sm_count_cached();
-    const int64_t need = (groups + FIELD_WARPS - 1) / FIELD_WARPS;
-    if (grid > need) grid = need;
-    if (grid < 1) grid = 1;
+    const int64_t warps = grid * FIELD_WARPS, share = (ntiles + warps - 1) / warps, rounds = (share + 31) / 32;
+    F.group = (int)((share + rounds - 1) / rounds);
+    const int64_t groups = (ntiles + F.group - 1) / F.group;
+    if (grid > groups) grid = groups;
     kern<<<(unsigned)grid, FIELD_WARPS * 32, smem, st>>>(a, F);
     return rd_check_launch("field_kernel");
 }
