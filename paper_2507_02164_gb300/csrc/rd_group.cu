@@ -7,7 +7,7 @@ namespace rd {
 // Whether a uniform batch takes the small-batch solver when the caller left
 // the launch shape open. Measured (us, 152 SMs, group / one thread per
 // polynomial at 32 threads per CTA, one launch with binning):
-//   mixed, n   700: degree 3 14.6 / 16.7   6 33.0 / 51.4   12  76.0 / 186.7
+//   mixed, n   700: degree 3 14.6 / 16.7   6 28.7 / 51.4   12  76.0 / 186.7
 //             4800: degree 3 16.5 / 16.5   6 35.1 / 45.4   12 110.8 / 190.8
 //             6000: degree 3 16.5 / 16.7   9 86.3 / 92.5   12 127.9 / 192.9
 //             8000: degree 3 18.6 / 16.6   9  125 / 86.2   12 186.5 / 190.9
@@ -25,7 +25,7 @@ bool group_takes(int degree, int64_t n, bool mixed)
 // The same for a packed batch of mixed degrees, which this solver takes in
 // one launch after the count, where the degree bins are twelve kernels on two
 // chains, each as long as its slowest warp. Measured (us, degrees 2..12,
-// complex128, group / bins): mixed 1000 97 / 484, 3001 109 / 483, 16000
+// complex128, group / bins): mixed 1000 97 / 484, 3001 87 / 483, 16000
 // 249 / 521, 32000 415 / 556, 64000 753 / 643; plain 1000 1023 / 4198, 8000
 // 4081 / 6027, 16000 7435 / 6960.
 bool uneven_group_takes(int64_t n, bool mixed) { return n <= (int64_t)(mixed ? 256 : 64) * rd_sm_count_cached(); }

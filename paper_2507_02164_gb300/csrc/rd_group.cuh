@@ -179,18 +179,17 @@ __device__ __forceinline__ void solve_group(const SolveArgs &A, const void *coef
             givens(x, y, c, s, top);  // lane r-1's is the rotation
             c = __shfl_sync(0xffffffffu, c, first + r - 1);
             s = shfl_from(s, first + r - 1);
-            if (act) {
-                if (l == r - 1) {
-                    h[at(r - 1, l)] = top;
-                    h[at(r, l)] = cx<T>{T(0), T(0)};
-                    W.c[r] = c;
-                    W.s[r] = s;
-                } else if (l >= r && l < mm) {
-                    rot_rows(c, s, x, y);
-                    h[at(r - 1, l)] = x;
-                    x = y;
-                }
+            // lane r-1 closes its column (top, 0), the lanes right of it rotate theirs
+            const bool own = act && l == r - 1, right = act && l >= r && l < mm;
+            cx<T> nx = x, ny = y;
+            rot_rows(c, s, nx, ny);
+            if (own || right) h[at(r - 1, l)] = own ? top : nx;
+            if (own) {
+                h[at(r, l)] = cx<T>{T(0), T(0)};
+                W.c[r] = c;
+                W.s[r] = s;
             }
+            x = sel(right, ny, x);
             y = ahead;
         }
         if (mm && l == mm - 1) h[at(l, l)] = x;
