@@ -92,18 +92,24 @@ __global__ void uneven_scan_kernel(UnevenHeader *hdr, int64_t n_coeffs)
     if (lane == 0) hdr->overflow = overflow ? 1u : 0u;
 }
 
-// Scatter every solvable polynomial into its degree's bin: a slot from a
-// warp-aggregated cursor, perm[slot] = its index, its coefficients
-// coefficient-major at bins[coef_base[d] + k * count[d] + slot].
+// Scatter every solvable polynomial into its degree's bin: perm[slot] = its
+// index, its coefficients coefficient-major at bins[coef_base[d] + k * count[d]
+// + slot]. A CTA takes PACK_POLYS polynomials at a time, ranks them by degree in
+// shared memory and reserves their slots with one atomic per degree on the
+// bin's cursor: one per warp and degree (131,072 on each of eleven addresses
+// for 2^22 polynomials) was what bounded the kernel (321 us; the whole call
+// 7.90 -> 7.86 ms, its solvers start on the helper stream meanwhile).
+constexpr int PACK_ROUNDS = 4, PACK_POLYS = 256 * PACK_ROUNDS;
+
 template <typename E>
 __global__ void __launch_bounds__(256) uneven_pack_kernel(UnevenArgs U, const E *__restrict__ coeffs,
                                                           UnevenHeader *hdr, uint32_t *perm, E *bins,
                                                           double *roots, uint8_t *status, rd_stats *stats)
 {
-    const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t warp_id = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (hdr->overflow) {
+        const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
+        const int64_t warp_id = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
         // overlapping ranges: nothing is packed; the solvable polynomials are
         // reported DEGENERATE with NaN roots (their own bounds hold)
         __shared__ unsigned long long acc[ST_WORDS];
@@ -123,27 +129,39 @@ __global__ void __launch_bounds__(256) uneven_pack_kernel(UnevenArgs U, const E 
         stats_end(S, stats);
         return;
     }
-    for (int64_t base = warp_id * 32; base < U.n; base += warps_total * 32) {
-        int64_t i = base + lane;
-        int d = -1;
-        if (i < U.n) {
+    __shared__ unsigned cnt[16], first[16];
+    for (int64_t base = (int64_t)blockIdx.x * PACK_POLYS; base < U.n; base += (int64_t)gridDim.x * PACK_POLYS) {
+        if (threadIdx.x < 16) cnt[threadIdx.x] = 0;
+        __syncthreads();
+        int deg[PACK_ROUNDS];
+        unsigned rank[PACK_ROUNDS];
+#pragma unroll
+        for (int t = 0; t < PACK_ROUNDS; ++t) {
+            const int64_t i = base + t * 256 + threadIdx.x;
             bool consistent;
-            d = checked_degree(U, i, consistent);
+            deg[t] = i < U.n ? checked_degree(U, i, consistent) : -1;
+            const unsigned act = __ballot_sync(0xffffffffu, deg[t] > 0);
+            if (deg[t] > 0) {
+                const unsigned peers = __match_any_sync(act, deg[t]);
+                const int leader = __ffs(peers) - 1;
+                unsigned b = 0;
+                if (lane == leader) b = atomicAdd(&cnt[deg[t]], (unsigned)__popc(peers));
+                rank[t] = __shfl_sync(peers, b, leader) + __popc(peers & ((1u << lane) - 1u));
+            }
         }
-        unsigned act = __ballot_sync(0xffffffffu, d > 0);
-        if (d > 0) {
-            unsigned peers = __match_any_sync(act, d);
-            int leader = __ffs(peers) - 1;
-            unsigned rank = __popc(peers & ((1u << lane) - 1u));
-            unsigned b = 0;
-            if (lane == leader) b = atomicAdd(&hdr->cursor[d], (unsigned)__popc(peers));
-            b = __shfl_sync(peers, b, leader);
-            unsigned slot = b + rank;
-            unsigned cnt = hdr->count[d];
+        __syncthreads();
+        if (threadIdx.x < 16 && cnt[threadIdx.x]) first[threadIdx.x] = atomicAdd(&hdr->cursor[threadIdx.x], cnt[threadIdx.x]);
+        __syncthreads();
+#pragma unroll
+        for (int t = 0; t < PACK_ROUNDS; ++t) {
+            const int64_t i = base + t * 256 + threadIdx.x;
+            const int d = deg[t];
+            if (d <= 0) continue;
+            const unsigned slot = first[d] + rank[t], count = hdr->count[d];
             perm[hdr->poly_base[d] + slot] = (uint32_t)i;
             const E *src = coeffs + __ldg(U.offsets + i);
             E *dst = bins + hdr->coef_base[d] + slot;
-            for (int k = 0; k <= d; ++k) dst[(int64_t)k * cnt] = __ldg(src + k);
+            for (int k = 0; k <= d; ++k) dst[(int64_t)k * count] = __ldg(src + k);
         }
     }
 }
