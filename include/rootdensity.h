@@ -272,14 +272,14 @@ int rd_pointer_is_device_accessible(const void *p);
  *             degree); see rd_uneven_tuning
  * n < 2^32 and n_coeffs <= 2^40 (RD_EINVAL otherwise;
  * rd_uneven_workspace_bytes returns 0 outside these limits). Only enqueues
- * work (16 kernel launches): the degree bins run as two chains, one on
- * `stream` and one on a helper stream of the calling host thread, forked from
- * and joined back to `stream` with events, so the whole call can be captured
- * in a CUDA graph (as two parallel branches) and `stream` orders everything
- * before and after it. The first call on a device from a host thread creates
- * the helper stream and its two events; make that call outside capture.
+ * work (16 kernel launches): the degree bins run as 4 chains (12 for a small
+ * batch), one on `stream` and the others on helper streams of the calling host
+ * thread, forked from and joined back to `stream` with events, so the whole call
+ * can be captured in a CUDA graph (as parallel branches) and `stream` orders
+ * everything before and after it. The first call on a device from a host thread
+ * creates the helper streams and their events; make that call outside capture.
  * (With the launch shape open -- no tuning, no shape in params -- a small batch
- * is solved without bins, in 3 launches on `stream` and no helper stream; a
+ * is solved without bins, in 3 launches on `stream` alone; a
  * degree whose tuning entries are all 0 keeps its shape open.) */
 typedef struct {
     /* Launch shape of each degree bin's solve kernel, indexed by the degree
@@ -309,7 +309,7 @@ int rd_roots_uneven(const void *coeffs, rd_dtype dtype, const uint8_t *degrees, 
  * would synchronise the device, deployments with a device-memory budget
  * fixed in advance. It behaves like rd_roots_uneven (same arguments without
  * ws/ws_bytes, same results; its degree bins all run on `stream`, so it makes
- * no helper stream either) but uses a scratch array of
+ * no helper streams either) but uses a scratch array of
  * RD_STATIC_SCRATCH_BYTES bytes built into the library: that memory is held
  * on every GPU that loads the library until the process exits, and the call
  * itself allocates and frees nothing.

@@ -23,12 +23,12 @@ bool group_takes(int degree, int64_t n, bool mixed)
 }
 
 // The same for a packed batch of mixed degrees, which this solver takes in
-// one launch after the count, where the degree bins are twelve kernels on two
-// chains, each as long as its slowest warp. Measured (us, degrees 2..12,
-// complex128, group / bins): mixed 1000 97 / 484, 3001 87 / 483, 16000
-// 249 / 521, 32000 415 / 556, 64000 753 / 643; plain 1000 1023 / 4198, 8000
-// 4081 / 6027, 16000 7435 / 6960.
-bool uneven_group_takes(int64_t n, bool mixed) { return n <= (int64_t)(mixed ? 256 : 64) * rd_sm_count_cached(); }
+// one launch after the count, where the degree bins are twelve kernels side by
+// side, as long as the slowest warp of them. Measured (us, degrees 2..12,
+// complex128, group / bins): mixed 3001 87 / 250, 8000 148 / 290, 16000 236 / 331,
+// 20000 279 / 335, 24000 321 / 341, 30000 383 / 333 (compensated 20000 280 / 296,
+// 24000 320 / 296); plain 2000 1319 / 2172, 4000 2354 / 2351, 8000 4207 / 2587.
+bool uneven_group_takes(int64_t n, bool mixed) { return n <= (int64_t)(mixed ? 144 : 24) * rd_sm_count_cached(); }
 
 template <int G, typename In, int MODE>
 static int launch_group_n(int degree, const SolveArgs &a, cudaStream_t st)

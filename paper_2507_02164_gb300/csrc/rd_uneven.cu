@@ -167,68 +167,92 @@ __global__ void __launch_bounds__(256) uneven_pack_kernel(UnevenArgs U, const E 
 }
 
 namespace {
-// The helper stream and its two events, per device, owned by one host thread
-// and released when that thread exits (errors ignored: at process exit the
-// runtime may already be gone).
+// The helper streams, the fork event and a join event for each, per device,
+// owned by one host thread and released when that thread exits (errors
+// ignored: at process exit the runtime may already be gone).
 struct ForkState {
-    int device = -1;
-    cudaStream_t side = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
-    ~ForkState()
+    cudaStream_t side[UNEVEN_SIDES] = {};
+    cudaEvent_t fork = nullptr, join[UNEVEN_SIDES] = {};
+    void release()
     {
         if (fork) cudaEventDestroy(fork);
-        if (join) cudaEventDestroy(join);
-        if (side) cudaStreamDestroy(side);
+        for (int k = 0; k < UNEVEN_SIDES; ++k) {
+            if (join[k]) cudaEventDestroy(join[k]);
+            if (side[k]) cudaStreamDestroy(side[k]);
+        }
     }
+    void forget()
+    {
+        fork = nullptr;
+        for (int k = 0; k < UNEVEN_SIDES; ++k) {
+            join[k] = nullptr;
+            side[k] = nullptr;
+        }
+    }
+    ~ForkState() { release(); }
 };
 thread_local ForkState g_fork[64];
 }  // namespace
 
-int uneven_fork(cudaStream_t st, cudaStream_t *side, cudaEvent_t *fork, cudaEvent_t *join, bool retry)
+// The calling host thread's handles on the current device, made on its first call.
+static int uneven_handles(ForkState **out)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return rd_set_error(RD_ECUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
     if (dev < 0 || dev >= 64) return rd_set_error(RD_EUNSUPPORTED, "device index %d above 63", dev);
     ForkState &f = g_fork[dev];
-    if (!f.side) {
-        // all three or none: a partial failure releases what it made
-        cudaStream_t s = nullptr;
-        cudaEvent_t a = nullptr, b = nullptr;
-        if ((e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking)) != cudaSuccess ||
-            (e = cudaEventCreateWithFlags(&a, cudaEventDisableTiming)) != cudaSuccess ||
-            (e = cudaEventCreateWithFlags(&b, cudaEventDisableTiming)) != cudaSuccess) {
-            if (a) cudaEventDestroy(a);
-            if (s) cudaStreamDestroy(s);
-            return rd_set_error(RD_ECUDA, "uneven helper stream: %s (the first call on a device from a host thread "
-                                          "creates it; make that call outside stream capture)",
+    if (!f.fork) {
+        // all or none: a partial failure releases what it made
+        e = cudaEventCreateWithFlags(&f.fork, cudaEventDisableTiming);
+        for (int k = 0; k < UNEVEN_SIDES && e == cudaSuccess; ++k) {
+            e = cudaStreamCreateWithFlags(&f.side[k], cudaStreamNonBlocking);
+            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&f.join[k], cudaEventDisableTiming);
+        }
+        if (e != cudaSuccess) {
+            f.release();
+            f.forget();
+            return rd_set_error(RD_ECUDA, "uneven helper streams: %s (the first call on a device from a host thread "
+                                          "creates them; make that call outside stream capture)",
                                 cudaGetErrorString(e));
         }
-        f.side = s;
-        f.fork = a;
-        f.join = b;
-        f.device = dev;
     }
-    if ((e = cudaEventRecord(f.fork, st)) != cudaSuccess || (e = cudaStreamWaitEvent(f.side, f.fork, 0)) != cudaSuccess) {
+    *out = &f;
+    return RD_OK;
+}
+
+int uneven_fork(cudaStream_t st, int sides, UnevenFork *out, bool retry)
+{
+    ForkState *state = nullptr;
+    int rc = uneven_handles(&state);
+    if (rc) return rc;
+    ForkState &f = *state;
+    cudaError_t e;
+    e = cudaEventRecord(f.fork, st);
+    for (int k = 0; k < sides && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(f.side[k], f.fork, 0);
+    if (e != cudaSuccess) {
         // handles made before a cudaDeviceReset are gone: forget them (they
         // cannot be destroyed any more) and make new ones, once
         if (e != cudaErrorInvalidResourceHandle || retry) return rd_set_error(RD_ECUDA, "uneven fork: %s", cudaGetErrorString(e));
         cudaGetLastError();
-        f.side = nullptr;
-        f.fork = f.join = nullptr;
-        return uneven_fork(st, side, fork, join, true);
+        f.forget();
+        return uneven_fork(st, sides, out, true);
     }
-    *side = f.side;
-    *fork = f.fork;
-    *join = f.join;
+    out->sides = sides;
+    for (int k = 0; k < sides; ++k) {
+        out->side[k] = f.side[k];
+        out->join[k] = f.join[k];
+    }
     return RD_OK;
 }
 
-int uneven_join(cudaStream_t st, cudaStream_t side, cudaEvent_t join)
+int uneven_join(cudaStream_t st, const UnevenFork &f)
 {
-    cudaError_t e;
-    if ((e = cudaEventRecord(join, side)) != cudaSuccess || (e = cudaStreamWaitEvent(st, join, 0)) != cudaSuccess)
-        return rd_set_error(RD_ECUDA, "uneven join: %s", cudaGetErrorString(e));
+    for (int k = 0; k < f.sides; ++k) {
+        cudaError_t e;
+        if ((e = cudaEventRecord(f.join[k], f.side[k])) != cudaSuccess || (e = cudaStreamWaitEvent(st, f.join[k], 0)) != cudaSuccess)
+            return rd_set_error(RD_ECUDA, "uneven join: %s", cudaGetErrorString(e));
+    }
     return RD_OK;
 }
 
@@ -267,7 +291,16 @@ int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const
     if ((rc = rd_check_launch("uneven_count_kernel"))) return rc;
     bool all_open = true;
     for (int d = 1; d <= UNEVEN_MAX_DEG; ++d) all_open &= open_shape[d];
-    if (all_open && uneven_group_takes(n, mixed)) return launch_uneven_group(a, dt, U, L.hdr, mixed, st);
+    if (all_open && uneven_group_takes(n, mixed)) {
+        // the first call of a host thread makes the helper streams whatever its
+        // size, so that a larger batch can be captured after it
+        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+        if (fork && cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) {
+            ForkState *state = nullptr;
+            if ((rc = uneven_handles(&state))) return rc;
+        }
+        return launch_uneven_group(a, dt, U, L.hdr, mixed, st);
+    }
     int bins_pw[16];
     const bool split = uneven_split_takes(n, mixed, a.polish_mode);
     for (int d = 0; d < 16; ++d) bins_pw[d] = split && open_shape[d] && d >= 4 && d <= UNEVEN_MAX_DEG ? UNEVEN_SPLIT : pw[d];

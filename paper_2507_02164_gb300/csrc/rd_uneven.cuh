@@ -91,12 +91,18 @@ inline UnevenLayout uneven_layout(void *ws, int64_t n)
     return L;
 }
 
-// Fork: a helper stream of the calling host thread on the current device
-// (created on its first use, non-blocking) made to wait for `st`; join:
-// `st` made to wait for the helper. Both only record and wait on events, so
-// they can be captured into a CUDA graph (as two parallel branches).
-int uneven_fork(cudaStream_t st, cudaStream_t *side, cudaEvent_t *fork, cudaEvent_t *join, bool retry = false);
-int uneven_join(cudaStream_t st, cudaStream_t side, cudaEvent_t join);
+// Fork: helper streams of the calling host thread on the current device
+// (created on their first use, non-blocking) made to wait for `st`; join:
+// `st` made to wait for all of them. Both only record and wait on events, so
+// they can be captured into a CUDA graph (as parallel branches).
+constexpr int UNEVEN_SIDES = 11;
+struct UnevenFork {
+    int sides;  // streams forked
+    cudaStream_t side[UNEVEN_SIDES];
+    cudaEvent_t join[UNEVEN_SIDES];
+};
+int uneven_fork(cudaStream_t st, int sides, UnevenFork *out, bool retry = false);
+int uneven_join(cudaStream_t st, const UnevenFork &f);
 
 // Large bins, FP64 polish: the split-register solver (rd_solve_split.cuh).
 int launch_uneven_split(int degree, rd_dtype dt, const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets,
