@@ -44,13 +44,17 @@ W_PIX, H_PIX = 1920, 1080
 E2E_CHUNK_LOG2 = 22
 # ncu summary of each form of the headline kernel, with the source hash it was taken on
 PROFILE_SUMMARY = {"one_role": os.path.join(ROOT, "profiles", "solve_mixed_littlewood_deg6.md"),
-                   "ws": os.path.join(ROOT, "profiles", "solve_ws_littlewood_deg6.md")}
+                   "ws": os.path.join(ROOT, "profiles", "solve_ws_littlewood_deg6.md"),
+                   "split": os.path.join(ROOT, "profiles", "solve_split_littlewood_deg6.md")}
 # Each solve kernel's code and its launch (the .cu files only dispatch to them); an ncu
 # traffic figure is valid only for the source it was taken on.
 KERNEL_SOURCES = {"one_role": ["paper_2507_02164_gb300/csrc/rd_solve.cuh", "paper_2507_02164_gb300/csrc/rd_common.cuh",
                                "paper_2507_02164_gb300/csrc/rd_solve_launch.cuh"],
                   "ws": ["paper_2507_02164_gb300/csrc/rd_solve.cuh", "paper_2507_02164_gb300/csrc/rd_common.cuh",
-                         "paper_2507_02164_gb300/csrc/rd_solve_ws.cuh"]}  # device code; launch: rd_solve_ws_launch.cuh
+                         "paper_2507_02164_gb300/csrc/rd_solve_ws.cuh"],  # device code; launch: rd_solve_ws_launch.cuh
+                  "split": ["paper_2507_02164_gb300/csrc/rd_solve.cuh", "paper_2507_02164_gb300/csrc/rd_common.cuh",
+                            "paper_2507_02164_gb300/csrc/rd_solve_ws.cuh",
+                            "paper_2507_02164_gb300/csrc/rd_solve_split.cuh"]}
 FP32_LANES_PER_SM = 128   # FP32 FMA lanes per SM (4 SMSPs x 32)
 FP64_FMA_PER_SM_CLK = 2   # FP64 FMA per SM per clock: 1.25 TFLOP/s / (152 SMs x 2 flop x 2.07 GHz)
 
@@ -84,7 +88,7 @@ def kernel_source_hash(form: str = "one_role") -> str:
 
 
 def profiled_traffic(form: str = "one_role"):
-    """Per-launch DRAM bytes of the solve kernel (form "one_role" or "ws") from
+    """Per-launch DRAM bytes of the solve kernel (form "one_role", "ws" or "split") from
     the committed ncu summary, or None when the summary is missing or was
     taken on other kernel source."""
     try:
@@ -489,11 +493,13 @@ def run_ours(args, rank: int, world: int, local_rank: int):
     f32, f64 = algorithmic_flops(st_mx)
     t_k = kern_mx * 1e-3
     frac32, frac64 = f32 / p32 / t_k, f64 / p64 / t_k
-    traffic = profiled_traffic("ws" if tuned["mixed"]["degrees"][str(DEGREE)].get("polish_warps", 0) else "one_role")
-    pw = tuned["mixed"]["degrees"][str(DEGREE)].get("polish_warps", 0)
-    blk = tuned["mixed"]["degrees"][str(DEGREE)]["block"]
-    kernel_name = (f"rd::solve_ws_kernel<6, float2> (warp-specialised: {pw} polish warps of {blk // 32})" if pw
-                   else "rd::solve_kernel<6, float, float2, MIXED>")
+    shape = tuned["mixed"]["degrees"][str(DEGREE)]
+    pw, blk = shape.get("polish_warps", 0), shape["block"]
+    form = "split" if shape.get("open", {}).get("faster") else ("ws" if pw else "one_role")
+    traffic = profiled_traffic(form)
+    kernel_name = {"split": "rd::solve_split_kernel<6, float2> (warp-specialised, register shares per role)",
+                   "ws": f"rd::solve_ws_kernel<6, float2> (warp-specialised: {pw} polish warps of {blk // 32})",
+                   "one_role": "rd::solve_kernel<6, float, float2, MIXED>"}[form]
     roofline = {
         "bound": "alu", "kernel": kernel_name,
         "achieved": (f32 + f64 * p32 / p64) / t_k / 1e12, "peak": p32 / 1e12, "unit": "TFLOP/s",

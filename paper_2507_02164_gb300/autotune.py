@@ -7,7 +7,10 @@ threads per CTA, resident CTAs per SM, and for the mixed mode the
 warp-specialised CTAs (params.polish_warps: some warps polish what the others
 sweep). The fastest shape serves uniform batches; the fastest shape without
 warp specialisation serves the uneven-degree bins, whose per-degree kernels
-have no warp-specialised form. This module calls it once per degree and
+have no warp-specialised form. An open shape (every launch field 0: the library
+picks the form by degree and batch size, forms that no explicit shape names
+among them) is timed against the fastest explicit one here and kept where it
+wins. This module calls the tuner once per degree and
 caches the results in a JSON file keyed by GPU, mode, storage type, probe
 size and a hash of the library's sources, so that a process tunes once and a
 rebuilt library is tuned again.
@@ -24,7 +27,7 @@ import torch
 from . import _native as N
 from . import api, build
 
-CACHE_FORMAT = 5  # table rows [lanes, block, ctas_per_sm, polish_warps, ms]
+CACHE_FORMAT = 6  # table rows [lanes, block, ctas_per_sm, polish_warps, ms]; "open": {"ms", "best_ms", "faster"}
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "rootdensity_tuning.json")
 TABLE_CAP = 64
 
@@ -50,6 +53,33 @@ def tune_degree(degree: int, mode: str = "mixed", dtype=torch.complex64, n: int 
     return res, (_entry(t.best), float(t.best.ms)), (_entry(t.one_role), float(t.one_role.ms))
 
 
+def time_open_shape(degree: int, mode: str, dtype, n: int, polish: str, best: tuple, reps: int = 5) -> dict:
+    """{"ms": the open shape, "best_ms": the explicit shape `best`, "faster": whether
+    the open one wins}, medians over one complex-Gaussian probe batch."""
+    dev = torch.device("cuda", torch.cuda.current_device())
+    real = torch.float32 if dtype == torch.complex64 else torch.float64
+    g = torch.Generator(device=dev).manual_seed(977 + degree)
+    co = torch.complex(*torch.randn((2, degree + 1, n), generator=g, device=dev, dtype=real))
+    hist, win = api.new_hist(1920, 1080, dev), api.Window(-3.0, 3.0, -1.6875, 1.6875)
+    extra = {"polish_mode": POLISH[polish]} if mode == "mixed" else {}
+    lanes, block, cps, pw = best
+    shapes = (api.params(mode, **extra),
+              api.params(mode, lanes=lanes, block=block, ctas_per_sm=cps, polish_warps=pw, **extra))
+    out = []
+    for p in shapes:
+        api.roots_density(co, win, hist, mode=mode, params_=p)
+        times = []
+        for _ in range(reps):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            api.roots_density(co, win, hist, mode=mode, params_=p)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        out.append(sorted(times)[reps // 2])
+    return {"ms": out[0], "best_ms": out[1], "faster": out[0] < out[1]}
+
+
 def cache_key(mode: str, dtype, n: int, polish: str = "fp64") -> str:
     name = torch.cuda.get_device_name()
     kind = "c64" if dtype == torch.complex64 else "c128"
@@ -71,7 +101,7 @@ def tune(mode: str = "mixed", dtype=torch.complex64, degrees=range(1, 13), n: in
     mode and polish, storage type, probe size and library sources) are not
     re-measured.
     Returns {"degrees": {d: {"lanes", "block", "ctas_per_sm", "polish_warps",
-    "ms", "one_role": {"lanes", "block", "ctas_per_sm", "ms"}, "table"}},
+    "ms", "one_role": {"lanes", "block", "ctas_per_sm", "ms"}, "open", "table"}},
     "seconds": time spent measuring, "probe_polys": n}."""
     key = cache_key(mode, dtype, n, polish)
     cache = load(cache_path) if cache_path else {}
@@ -84,6 +114,7 @@ def tune(mode: str = "mixed", dtype=torch.complex64, degrees=range(1, 13), n: in
         entry[str(d)] = {"lanes": best[0], "block": best[1], "ctas_per_sm": best[2], "polish_warps": best[3],
                          "ms": ms,
                          "one_role": {"lanes": one[0], "block": one[1], "ctas_per_sm": one[2], "ms": one_ms},
+                         "open": time_open_shape(d, mode, dtype, n, polish, best),
                          "table": [[la, b, c, pw, t] for (la, b, c, pw), t in sorted(res.items())]}
     spent = time.perf_counter() - t0
     if cache_path:
@@ -103,9 +134,12 @@ UNEVEN_WS_MAX_DEG = 8  # the uneven bins have a warp-specialised form up to this
 def uneven_tuning(result: dict):
     """rd_uneven_tuning (per degree) from a tune() result: each degree's
     fastest shape where the bins have it (the warp-specialised form up to
-    degree 8), else its fastest one-role shape."""
+    degree 8), else its fastest one-role shape; left open (all 0) where the open
+    shape won."""
     deg = {}
     for d, e in result["degrees"].items():
+        if e.get("open", {}).get("faster"):
+            continue
         if int(d) <= UNEVEN_WS_MAX_DEG and e.get("polish_warps", 0) > 0:
             deg[d] = {"block": e["block"], "ctas_per_sm": 0, "lanes": 1, "polish_warps": e["polish_warps"]}
         else:
@@ -119,8 +153,10 @@ def uneven_tuning(result: dict):
 
 def degree_params(result: dict, degree: int, mode: str = "mixed", polish: str = "fp64"):
     """rd_params for a uniform batch of `degree` from a tune() result (made
-    with the same polish)."""
+    with the same polish): the open shape where it won."""
     e = result["degrees"][str(degree)]
     extra = {"polish_mode": POLISH[polish]} if mode == "mixed" else {}
+    if e.get("open", {}).get("faster"):
+        return api.params(mode, **extra)
     return api.params(mode, block=e["block"], ctas_per_sm=e["ctas_per_sm"], lanes=e["lanes"],
                       polish_warps=e.get("polish_warps", 0), **extra)
