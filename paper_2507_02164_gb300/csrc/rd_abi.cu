@@ -139,7 +139,7 @@ bool shape_open(const rd_params &p)
     return p.block == 0 && p.ctas_per_sm == 0 && p.lanes == 0 && p.polish_warps == 0 && p.ring_slots == 0;
 }
 
-// The FP64 polish of a large enough batch takes the split-register
+// A large enough batch takes the split-register
 // warp-specialised solver (rd_solve_split.cuh). Measured on complex-Gaussian
 // polynomials (us, 152 SMs), split against the best other form:
 //   degree     n 40,000     60,000     80,000    100,003    150,000    2^19
@@ -152,32 +152,34 @@ bool shape_open(const rd_params &p)
 //   10           220 / 256  234 / 276  328 / 399  344 / 423  470 / 584  1506 / 1996
 //   12           342 / 410  409 / 453  562 / 644  626 / 707  874 / 983  2811 / 3229
 // (25,000: 9 116 / 112, 12 234 / 211). 2^24 Littlewood polynomials: 15.9 against
-// 17.3 ms.
+// 17.3 ms. Compensated polish (complex64; complex128 gains up to 6 % more):
+//   degree     n 40,000     60,000     80,000    100,003    150,000    300,007     2^19
+//    7            90 / 70   103 / 109  133 / 123  146 / 143  195 / 193  375 / 396   652 / 711
+//    8           114 / 92   132 / 145  168 / 164  189 / 194  259 / 266  512 / 560   875 / 1011
+//    9           144 / 148  165 / 172  216 / 233  240 / 265  325 / 364  625 / 735  1069 / 1305
+//   10           176 / 187  204 / 213  265 / 297  296 / 339  392 / 458  754 / 929  1286 / 1621
+//   11           226 / 246  268 / 261  349 / 374  396 / 394  526 / 546  997 / 1101 1672 / 1911
+// (25,000: 9 100 / 92, 11 141 / 138).
 bool split_takes(int degree, rd_dtype dtype, int64_t n, bool mixed, int polish_mode)
 {
-    if (!mixed || polish_mode != RD_POLISH_FP64 || degree < 4) return false;
+    if (!mixed || degree < 4) return false;
     const int64_t per_sm = n / rd_sm_count_cached();
+    if (polish_mode == RD_POLISH_DF) return degree >= 7 && degree <= 11 && per_sm >= (degree == 7 ? 1536 : (degree == 8 ? 640 : 256));
     if (degree == 4) return dtype == RD_C64 && per_sm >= 640;
     return per_sm >= (degree <= 6 ? 576 : (degree <= 8 ? 352 : 224));
 }
 
-// The launch shape of any other uniform batch too large for the small-batch
-// solver, when the caller left it open. Compensated polish: 256 threads against
-// 32 (warps that start together share the instruction cache) degree 6 300,000
-// 265 against 278 us, 2^20 904 against 973; 9 740 against 784; at 200,000 the last
-// wave's coarser grain costs more (10: 677 against 649); degrees 7 and 8, at 168
-// registers: 128 threads, three CTAs per SM (8 2^19 1019 against 1105 with
-// 256). Otherwise one warp per CTA, which spreads a ragged wave over all SMs:
-// plain degree 6 65,536 1164 against 1285 with 128 threads, degree 12 20,000 2359
-// against 3339; mixed degree 12 20,000 198 against 227; equal on full waves.
+// The launch shape of any other uniform batch, when the caller left it open: one
+// warp per CTA, which spreads a ragged wave over all SMs. Plain degree 6 65,536
+// 1164 us against 1285 with 128 threads, degree 12 20,000 2359 against 3339; mixed
+// degree 12 20,000 198 against 227; compensated 7 150,000 193 against 207 (128) and
+// 223 (256); equal on full waves. Except the compensated polish of degrees 5 and 6,
+// 256 threads (warps that start together share the instruction cache): degree 6
+// 300,000 265 against 278, 2^20 904 against 973, 2^19 448 against 470.
 void open_shape(rd_params &p, int degree, int64_t n, bool mixed)
 {
-    const int64_t per_sm = n / rd_sm_count_cached();
-    p.block = 32;
-    if (mixed && p.polish_mode == RD_POLISH_DF) {
-        if (degree == 7 || degree == 8) p.block = 128;
-        else if (degree >= 5 && per_sm >= 1536) p.block = 256;
-    }
+    const bool df = mixed && p.polish_mode == RD_POLISH_DF;
+    p.block = df && (degree == 5 || degree == 6) && n / rd_sm_count_cached() >= 1536 ? 256 : 32;
 }
 
 // Validate a tile clip (host struct, device arrays) for n polynomials.

@@ -1,5 +1,5 @@
-// rd_solve_split.cuh -- warp-specialised RD_MIXED solver with the FP64 polish
-// whose two roles have register shares of their own (setmaxnreg).
+// rd_solve_split.cuh -- warp-specialised RD_MIXED solver whose two roles have
+// register shares of their own (setmaxnreg).
 //
 // GB300's FP64 unit belongs to an SM sub-partition, takes 67.5 cycles per warp
 // instruction, and one warp with a single dependent chain keeps it busy. What
@@ -51,9 +51,32 @@ __host__ __device__ constexpr SplitShape split_shape(int n)
                      : SplitShape{8, 8, 40, 12};
 }
 
-template <int N>
+// The same for the compensated polish, whose work is FP32 like the sweeps':
+// what the split gives it is eight sweep warps with the registers they want
+// beside eight that need few, where the one-role kernel has 8 to 12 in all.
+// Measured as above (2^19, complex64; one role 7 711, 8 1010, 9 1302, 10 1620,
+// 11 1901, 12 2448):
+//   7: 8/8/72 652, 12/8/72 716, 8/12/64 774     8: 8/8/72 875, 12/8/72 919, 8/12/64 947
+//   9: 8/8/64 1069, 8/8/72 1074, 8/8/48 1088   10: 8/8/64 1286, 8/8/72 1303, 8/8/40 1347
+//  11: 8/8/40 1680, 8/8/48 1709, 8/8/56 1815, 8/8/64 1960 (the sweeps spill)
+// Degree 12 spills in every split (2614 the best), and 4 to 6 already have
+// sixteen warps in one role: not built.
+__host__ __device__ constexpr SplitShape split_shape_df(int n)
+{
+    return n <= 8    ? SplitShape{8, 8, 72, 24}
+           : n <= 10 ? SplitShape{8, 8, 64, 24}
+                     : SplitShape{8, 8, 40, 16};
+}
+
+// The degrees each polish is built for.
+__host__ __device__ constexpr bool split_built(int n, int mode)
+{
+    return mode == MODE_MIXED_DF ? n >= 7 && n <= 11 : n >= 4 && n <= 12;
+}
+
+template <int N, int MODE>
 struct Split {
-    static constexpr SplitShape shape = split_shape(N);
+    static constexpr SplitShape shape = MODE == MODE_MIXED_DF ? split_shape_df(N) : split_shape(N);
     static constexpr int SWEEP = shape.sweep, POLISH = shape.polish, POLISH_REGS = shape.polish_regs, SLOTS = shape.slots;
     static constexpr int THREADS = 32 * (SWEEP + POLISH);
     static constexpr int LAUNCH_REGS = 65536 / THREADS / 8 * 8;
@@ -62,32 +85,39 @@ struct Split {
     static_assert(POLISH_REGS % 8 == 0 && POLISH_REGS <= LAUNCH_REGS && LAUNCH_REGS <= SWEEP_REGS && SWEEP_REGS <= 256, "");
     static_assert(SWEEP * SWEEP_REGS + POLISH * POLISH_REGS <= (SWEEP + POLISH) * LAUNCH_REGS,
                   "the shares must fit the registers of the launch, or setmaxnreg.inc waits forever");
+    static_assert(split_built(N, MODE), "");
     static_assert(SLOTS > POLISH && SLOTS <= WS_MAX_SLOTS, "a polish warp keeps its slot until it has finished it");
 };
 
 // A polish warp's shared memory: lane-major, one 8- or 16-byte access per
 // lane and value, 256 or 512 contiguous bytes per warp.
-template <int N>
+template <int N, bool LO>
 struct LeanMem {
-    double2 ad[N + 1][32];  // coefficients in FP64 (complex128: scaled by a power of two)
-    double2 z[N][32];       // polished roots
-    float2 af[N + 1][32];   // coefficients in FP32
+    double2 ad[N + 1][32];              // coefficients in FP64 (complex128: scaled by a power of two)
+    double2 z[N][32];                   // polished roots
+    float2 af[N + 1][32];               // coefficients in FP32
+    float2 alo[LO ? N + 1 : 1][LO ? 32 : 1];  // what FP32 leaves of them (compensated polish, complex128)
 };
+template <typename In, int MODE>
+constexpr bool lean_lo = MODE == MODE_MIXED_DF && !std::is_same<In, float2>::value;
+template <int N, typename In, int MODE>
+constexpr size_t lean_bytes = (sizeof(LeanMem<N, lean_lo<In, MODE>>) + 15) / 16 * 16;
 
-template <int N>
+template <int N, typename In, int MODE>
 __host__ __device__ constexpr size_t split_smem_bytes()
 {
-    return ws_smem_bytes(N, Split<N>::SLOTS) + (size_t)Split<N>::POLISH * sizeof(LeanMem<N>);
+    return ws_smem_bytes(N, Split<N, MODE>::SLOTS) + (size_t)Split<N, MODE>::POLISH * lean_bytes<N, In, MODE>;
 }
 
-// finish_lane with the FP64 polish for the eigenvalues in `slot`, its
+// finish_lane (either polish) for the eigenvalues in `slot`, its
 // coefficients and roots in `mem`. All 32 lanes of the warp call it together;
 // the slot's eigenvalues are overwritten (by the FP32 copies of the roots).
-template <int N, typename In, class Map>
+template <int N, typename In, int MODE, class Map>
 __device__ __forceinline__ void finish_lean(const SolveArgs &A, const void *coeffs, int64_t n, int64_t i,
-                                            const Map &map, const CtaStats &S, WsSlot<N> &slot, LeanMem<N> &mem,
-                                            bool degenerate, bool not_conv)
+                                            const Map &map, const CtaStats &S, WsSlot<N> &slot,
+                                            LeanMem<N, lean_lo<In, MODE>> &mem, bool degenerate, bool not_conv)
 {
+    constexpr bool DF = MODE == MODE_MIXED_DF, LO = lean_lo<In, MODE>;
     constexpr bool C64 = std::is_same<In, float2>::value;
     const int lane = threadIdx.x & 31;
     const bool valid = i < n;
@@ -139,7 +169,9 @@ __device__ __forceinline__ void finish_lean(const SolveArgs &A, const void *coef
                 cx<double> a = ad(k);
                 a = {a.re * f, a.im * f};
                 mem.ad[k][lane] = make_double2(a.re, a.im);
-                mem.af[k][lane] = make_float2(d2f(a.re), d2f(a.im));
+                const cx<float> h = d2f(a);
+                mem.af[k][lane] = make_float2(h.re, h.im);
+                if constexpr (LO) mem.alo[k][lane] = make_float2(d2f(a.re - f2d(h.re)), d2f(a.im - f2d(h.im)));
             }
         }
         const float rtol = A.residual_tol > 0 ? (float)A.residual_tol : (float)(64.0 * N * 0x1p-53);
@@ -163,30 +195,50 @@ __device__ __forceinline__ void finish_lean(const SolveArgs &A, const void *coef
 #pragma unroll 1
         for (int j = 0; j < N; ++j) {
             cx<float> zf = eigenvalue(j);
-            cx<double> zj = f2d(zf);
-            float moved = CUDART_INF_F;
+            cx<double> zj;
+            bool good = false;
+            if constexpr (DF) {
+                cx<float> zl = {0.0f, 0.0f};
+                auto lo = [&](int k) -> cx<float> {
+                    if constexpr (LO) return {mem.alo[k][lane].x, mem.alo[k][lane].y};
+                    return {0.0f, 0.0f};
+                };
 #pragma unroll 1
-            for (int step = 0; step < A.polish_steps; ++step) {
-                asm volatile("" ::: "memory");  // the coefficients stay in shared memory
-                // p in FP64 and, in its shadow, p' in FP32
-                cx<double> p = ad(N);
-                cx<float> pf = af(N), dp = {0.0f, 0.0f};
+                for (int step = 0; step < A.polish_steps; ++step) {
+                    asm volatile("" ::: "memory");  // the coefficients stay in shared memory
+                    CompHorner ch(zf, af(N), lo(N));
 #pragma unroll
-                for (int k = N - 1; k >= 0; --k) {
-                    p = cfma(p, zj, ad(k));
-                    dp = cfma(dp, zf, pf);
-                    pf = cfma(pf, zf, af(k));
+                    for (int k = N - 1; k >= 0; --k) ch.step<LO>(af(k), lo(k));
+                    if (!ch.newton(zf, zl)) break;
+                    newton += 1;
                 }
-                const cx<float> dz = cdiv(d2f(p), dp);
-                if (!finite_c(dz)) break;
-                zj = sub(zj, f2d(dz));
-                zf = sub(zf, dz);
-                moved = abs1(dz);
-                newton += 1;
+                zj = {f2d(zf.re) + f2d(zl.re), f2d(zf.im) + f2d(zl.im)};
+            } else {
+                zj = f2d(zf);
+                float moved = CUDART_INF_F;
+#pragma unroll 1
+                for (int step = 0; step < A.polish_steps; ++step) {
+                    asm volatile("" ::: "memory");  // the coefficients stay in shared memory
+                    // p in FP64 and, in its shadow, p' in FP32
+                    cx<double> p = ad(N);
+                    cx<float> pf = af(N), dp = {0.0f, 0.0f};
+#pragma unroll
+                    for (int k = N - 1; k >= 0; --k) {
+                        p = cfma(p, zj, ad(k));
+                        dp = cfma(dp, zf, pf);
+                        pf = cfma(pf, zf, af(k));
+                    }
+                    const cx<float> dz = cdiv(d2f(p), dp);
+                    if (!finite_c(dz)) break;
+                    zj = sub(zj, f2d(dz));
+                    zf = sub(zf, dz);
+                    moved = abs1(dz);
+                    newton += 1;
+                }
+                const cx<float> zr = d2f(zj);
+                const float az = sqrtf(norm2(zr));
+                good = residual_certain(N, moved, abs1(sub(zr, zf)), az, weight(az), abs1(af(N)), rtol);
             }
-            const cx<float> zr = d2f(zj);
-            const float az = sqrtf(norm2(zr));
-            bool good = residual_certain(N, moved, abs1(sub(zr, zf)), az, weight(az), abs1(af(N)), rtol);
             if (!__all_sync(0xffffffffu, good || degenerate)) good = passes(horner(zj), zj);
             failed |= (good ? 0u : 1u) << j;
             mem.z[j][lane] = make_double2(zj.re, zj.im);
@@ -279,8 +331,13 @@ __device__ __forceinline__ void finish_lean(const SolveArgs &A, const void *coef
     }
     const unsigned nw = (degenerate ? 0u : newton) + extra, nr = (degenerate || !polish) ? 0u : (unsigned)N;
     S.add(ST_NEWTON, nw);
-    S.add(ST_F64, (8u * N + 2u) * nw + (8u * N + 4u) * nr);
-    S.add(ST_F32, (8u * N + 3u) * nw + (2u * N + 4u) * nr);
+    if constexpr (DF) {
+        S.add(ST_F64, (8u * N + 6u) * nr);
+        S.add(ST_F32, (66u * N + 50u) * nw + (2u * N + 4u) * nr);
+    } else {
+        S.add(ST_F64, (8u * N + 2u) * nw + (8u * N + 4u) * nr);
+        S.add(ST_F32, (8u * N + 3u) * nw + (2u * N + 4u) * nr);
+    }
     S.add(ST_POLYS, valid ? 1u : 0u);
 #pragma unroll
     for (int k = 0; k < 4; ++k) S.add(ST_STATUS0 + k, (valid && st == k) ? 1u : 0u);
@@ -326,14 +383,15 @@ __device__ __forceinline__ void finish_lean(const SolveArgs &A, const void *coef
 
 // One CTA of the split form over a coefficient-major batch (ws_cta's tasks
 // and ring): warps 0 .. POLISH-1 polish, the others sweep.
-template <int N, typename In, class Map>
+template <int N, typename In, int MODE, class Map>
 __device__ __forceinline__ void split_cta(const SolveArgs &A, const void *coeffs, int64_t n, const Map &map)
 {
-    using C = Split<N>;
+    using C = Split<N, MODE>;
+    using Lean = LeanMem<N, lean_lo<In, MODE>>;
     extern __shared__ __align__(16) unsigned char ws_smem[];
-    LeanMem<N> *lean = reinterpret_cast<LeanMem<N> *>(ws_smem);
-    WsCtl *ctl = reinterpret_cast<WsCtl *>(ws_smem + C::POLISH * sizeof(LeanMem<N>));
-    WsSlot<N> *ring = reinterpret_cast<WsSlot<N> *>(ws_smem + C::POLISH * sizeof(LeanMem<N>) + sizeof(WsCtl));
+    constexpr size_t lean_all = C::POLISH * lean_bytes<N, In, MODE>;
+    WsCtl *ctl = reinterpret_cast<WsCtl *>(ws_smem + lean_all);
+    WsSlot<N> *ring = reinterpret_cast<WsSlot<N> *>(ws_smem + lean_all + sizeof(WsCtl));
     __shared__ unsigned long long acc[ST_WORDS];
     if (threadIdx.x == 0) {
         ctl->sweep_ticket = 0;
@@ -359,7 +417,7 @@ __device__ __forceinline__ void split_cta(const SolveArgs &A, const void *coeffs
             const int64_t i = (b + (int64_t)k * G) * 32 + lane;
             cx<float> d[N];
             bool degenerate, not_conv;
-            sweep_lane<N, float, In, MODE_MIXED_FP64>(A, coeffs, n, i, S, d, degenerate, not_conv);
+            sweep_lane<N, float, In, MODE>(A, coeffs, n, i, S, d, degenerate, not_conv);
             if (!ws_put<N>(ctl, ring, C::SLOTS, k, d, degenerate, not_conv, abort_flag)) break;
         }
     } else {
@@ -378,26 +436,27 @@ __device__ __forceinline__ void split_cta(const SolveArgs &A, const void *coeffs
             WsSlot<N> &w = ring[slot];
             const bool degenerate = (w.degenerate >> lane) & 1u;
             const bool not_conv = (w.not_conv >> lane) & 1u;
-            finish_lean<N, In>(A, coeffs, n, i, map, S, w, lean[warp], degenerate, not_conv);
+            Lean &lean = *reinterpret_cast<Lean *>(ws_smem + warp * lean_bytes<N, In, MODE>);
+            finish_lean<N, In, MODE>(A, coeffs, n, i, map, S, w, lean, degenerate, not_conv);
             ws_publish(&ctl->state[slot], 2u * round + 2u);
         }
     }
     stats_end(S, A.stats);
 }
 
-template <int N, typename In>
-__global__ void __launch_bounds__(Split<N>::THREADS, 1) solve_split_kernel(SolveArgs A)
+template <int N, typename In, int MODE>
+__global__ void __launch_bounds__(Split<N, MODE>::THREADS, 1) solve_split_kernel(SolveArgs A)
 {
-    split_cta<N, In>(A, A.coeffs, A.n, UniformMap{{}, A.n});
+    split_cta<N, In, MODE>(A, A.coeffs, A.n, UniformMap{{}, A.n});
 }
 
 // The degree-N bin of a packed batch (its size is read on the device).
-template <int N, typename In>
-__global__ void __launch_bounds__(Split<N>::THREADS, 1)
+template <int N, typename In, int MODE>
+__global__ void __launch_bounds__(Split<N, MODE>::THREADS, 1)
     uneven_split_kernel(SolveArgs A, const UnevenHeader *hdr, const uint32_t *perm, const char *bins, const int64_t *offsets)
 {
     const PackedMap map{{}, perm + hdr->poly_base[N], offsets};
-    split_cta<N, In>(A, bins + (size_t)hdr->coef_base[N] * sizeof(In), hdr->count[N], map);
+    split_cta<N, In, MODE>(A, bins + (size_t)hdr->coef_base[N] * sizeof(In), hdr->count[N], map);
 }
 
 }  // namespace rd

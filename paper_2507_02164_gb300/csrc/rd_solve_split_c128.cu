@@ -5,7 +5,7 @@ namespace rd {
 
 int launch_solve_split_c128(int degree, const SolveArgs &a, cudaStream_t st)
 {
-    return launch_split_degree<double2>(degree, a, st);
+    return launch_split_degree<double2, MODE_MIXED_FP64>(degree, a, st);
 }
 
 }  // namespace rd

@@ -12,7 +12,7 @@ namespace rd {
 // the kernel was built with the registers per thread that its roles' shares
 // were added up against (a share above what the launch holds would wait
 // forever). Host calls outside any stream order, so a capture may follow.
-template <int N, typename Kern>
+template <int N, typename In, int MODE, typename Kern>
 static int split_ready(Kern kern, std::atomic<int> (&ready)[64])
 {
     int dev = 0;
@@ -21,71 +21,65 @@ static int split_ready(Kern kern, std::atomic<int> (&ready)[64])
     if (ready[dev].load()) return RD_OK;
     cudaFuncAttributes attr;
     if (cudaFuncGetAttributes(&attr, kern) != cudaSuccess) return rd_check_launch("cudaFuncGetAttributes(split kernel)");
-    if (attr.numRegs != Split<N>::LAUNCH_REGS)
+    if (attr.numRegs != Split<N, MODE>::LAUNCH_REGS)
         return rd_set_error(RD_EUNSUPPORTED, "split kernel of degree %d built with %d registers per thread, %d expected", N,
-                            attr.numRegs, Split<N>::LAUNCH_REGS);
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_smem_bytes<N>()) != cudaSuccess)
+                            attr.numRegs, Split<N, MODE>::LAUNCH_REGS);
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_smem_bytes<N, In, MODE>()) != cudaSuccess)
         return rd_check_launch("cudaFuncSetAttribute(split kernel)");
     ready[dev].store(1);
     return RD_OK;
 }
 
-template <int N, typename In>
+template <int N, typename In, int MODE>
 static int launch_split_n(const SolveArgs &a, cudaStream_t st)
 {
     static std::atomic<int> ready[64];
-    auto kern = solve_split_kernel<N, In>;
-    int rc = split_ready<N>(kern, ready);
+    auto kern = solve_split_kernel<N, In, MODE>;
+    int rc = split_ready<N, In, MODE>(kern, ready);
     if (rc) return rc;
     const int64_t tasks = (a.n + 31) / 32, sms = rd_sm_count_cached();
-    kern<<<(unsigned)(tasks < sms ? tasks : sms), Split<N>::THREADS, split_smem_bytes<N>(), st>>>(a);
+    kern<<<(unsigned)(tasks < sms ? tasks : sms), Split<N, MODE>::THREADS, split_smem_bytes<N, In, MODE>(), st>>>(a);
     return rd_check_launch("solve_split_kernel");
 }
 
-template <typename In>
-static int launch_split_degree(int degree, const SolveArgs &a, cudaStream_t st)
-{
-    switch (degree) {
-    case 4: return launch_split_n<4, In>(a, st);
-    case 5: return launch_split_n<5, In>(a, st);
-    case 6: return launch_split_n<6, In>(a, st);
-    case 7: return launch_split_n<7, In>(a, st);
-    case 8: return launch_split_n<8, In>(a, st);
-    case 9: return launch_split_n<9, In>(a, st);
-    case 10: return launch_split_n<10, In>(a, st);
-    case 11: return launch_split_n<11, In>(a, st);
-    case 12: return launch_split_n<12, In>(a, st);
-    default: return rd_set_error(RD_EUNSUPPORTED, "degree %d not built (4..12)", degree);
-    }
-}
-
-template <int N, typename In>
+template <int N, typename In, int MODE>
 static int launch_uneven_split_n(const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets, cudaStream_t st)
 {
     static std::atomic<int> ready[64];
-    auto kern = uneven_split_kernel<N, In>;
-    int rc = split_ready<N>(kern, ready);
+    auto kern = uneven_split_kernel<N, In, MODE>;
+    int rc = split_ready<N, In, MODE>(kern, ready);
     if (rc) return rc;
-    kern<<<rd_sm_count_cached(), Split<N>::THREADS, split_smem_bytes<N>(), st>>>(a, L.hdr, L.perm, L.bins, offsets);
+    kern<<<rd_sm_count_cached(), Split<N, MODE>::THREADS, split_smem_bytes<N, In, MODE>(), st>>>(a, L.hdr, L.perm, L.bins, offsets);
     return rd_check_launch("uneven_split_kernel");
 }
 
-template <typename In>
+// LAUNCH<N>() for the degree, one instance for each degree that is built.
+#define RD_SPLIT_CASE(D, LAUNCH, ...) \
+    case D: \
+        if constexpr (split_built(D, MODE)) return LAUNCH<D, In, MODE>(__VA_ARGS__); \
+        break;
+#define RD_SPLIT_DEGREES(LAUNCH, ...) \
+    switch (degree) { \
+        RD_SPLIT_CASE(4, LAUNCH, __VA_ARGS__) RD_SPLIT_CASE(5, LAUNCH, __VA_ARGS__) RD_SPLIT_CASE(6, LAUNCH, __VA_ARGS__) \
+        RD_SPLIT_CASE(7, LAUNCH, __VA_ARGS__) RD_SPLIT_CASE(8, LAUNCH, __VA_ARGS__) RD_SPLIT_CASE(9, LAUNCH, __VA_ARGS__) \
+        RD_SPLIT_CASE(10, LAUNCH, __VA_ARGS__) RD_SPLIT_CASE(11, LAUNCH, __VA_ARGS__) RD_SPLIT_CASE(12, LAUNCH, __VA_ARGS__) \
+    } \
+    return rd_set_error(RD_EUNSUPPORTED, "split solver: degree %d not built", degree);
+
+template <typename In, int MODE>
+static int launch_split_degree(int degree, const SolveArgs &a, cudaStream_t st)
+{
+    RD_SPLIT_DEGREES(launch_split_n, a, st)
+}
+
+template <typename In, int MODE>
 static int launch_uneven_split_degree(int degree, const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets,
                                       cudaStream_t st)
 {
-    switch (degree) {
-    case 4: return launch_uneven_split_n<4, In>(a, L, offsets, st);
-    case 5: return launch_uneven_split_n<5, In>(a, L, offsets, st);
-    case 6: return launch_uneven_split_n<6, In>(a, L, offsets, st);
-    case 7: return launch_uneven_split_n<7, In>(a, L, offsets, st);
-    case 8: return launch_uneven_split_n<8, In>(a, L, offsets, st);
-    case 9: return launch_uneven_split_n<9, In>(a, L, offsets, st);
-    case 10: return launch_uneven_split_n<10, In>(a, L, offsets, st);
-    case 11: return launch_uneven_split_n<11, In>(a, L, offsets, st);
-    case 12: return launch_uneven_split_n<12, In>(a, L, offsets, st);
-    default: return rd_set_error(RD_EUNSUPPORTED, "degree %d not built (4..12)", degree);
-    }
+    RD_SPLIT_DEGREES(launch_uneven_split_n, a, L, offsets, st)
 }
+
+#undef RD_SPLIT_DEGREES
+#undef RD_SPLIT_CASE
 
 }  // namespace rd

@@ -262,16 +262,17 @@ size_t uneven_workspace_bytes(int64_t n, int64_t n_coeffs, rd_dtype dt)
     return uneven_bytes(n, n_coeffs, dt == RD_C64 ? 8 : 16);
 }
 
-// Whether the degree bins 4 to 12 take the split-register solver
+// Whether the degree bins 4 to 12 (compensated polish 7 to 11) take the split-register solver
 // (rd_solve_split.cuh) where the caller left their launch shapes open. The
 // bins' sizes exist only on the device, so the line is drawn on n; each split
 // kernel takes whole SMs, so small bins lose the overlap of the two chains.
 // Measured (us, degrees 2..12, complex64, split / one role): 300,000 1030 / 930,
 // 2^19 1560 / 1430, 2^20 2385 / 2498, 2^22 7909 / 9357 (complex128 2574 / 2621,
-// 8702 / 9864).
+// 8702 / 9864). Compensated polish: 2^20 1932 / 1888, 1,500,000 2583 / 2658,
+// 2^22 6683 / 7323 (complex128 2196 / 2134, 2903 / 2978, 7572 / 8327).
 static bool uneven_split_takes(int64_t n, bool mixed, int polish_mode)
 {
-    return mixed && polish_mode == RD_POLISH_FP64 && n >= (int64_t)6144 * rd_sm_count_cached();
+    return mixed && n >= (int64_t)(polish_mode == RD_POLISH_DF ? 9216 : 6144) * rd_sm_count_cached();
 }
 
 int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const int64_t *offsets, int64_t n,
@@ -302,8 +303,9 @@ int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const
         return launch_uneven_group(a, dt, U, L.hdr, mixed, st);
     }
     int bins_pw[16];
-    const bool split = uneven_split_takes(n, mixed, a.polish_mode);
-    for (int d = 0; d < 16; ++d) bins_pw[d] = split && open_shape[d] && d >= 4 && d <= UNEVEN_MAX_DEG ? UNEVEN_SPLIT : pw[d];
+    const bool split = uneven_split_takes(n, mixed, a.polish_mode), df = a.polish_mode == RD_POLISH_DF;
+    const int first = df ? 7 : 4, last = df ? 11 : UNEVEN_MAX_DEG;
+    for (int d = 0; d < 16; ++d) bins_pw[d] = split && open_shape[d] && d >= first && d <= last ? UNEVEN_SPLIT : pw[d];
     pw = bins_pw;
     uneven_scan_kernel<<<1, 32, 0, st>>>(L.hdr, n_coeffs);
     if ((rc = rd_check_launch("uneven_scan_kernel"))) return rc;

@@ -104,7 +104,7 @@ struct UnevenFork {
 int uneven_fork(cudaStream_t st, int sides, UnevenFork *out, bool retry = false);
 int uneven_join(cudaStream_t st, const UnevenFork &f);
 
-// Large bins, FP64 polish: the split-register solver (rd_solve_split.cuh).
+// Large bins: the split-register solver (rd_solve_split.cuh).
 int launch_uneven_split(int degree, rd_dtype dt, const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets,
                         cudaStream_t st);
 constexpr int UNEVEN_SPLIT = -1;  // in launch_uneven_bins' pw[d]
@@ -118,7 +118,7 @@ bool uneven_group_takes(int64_t n, bool mixed);
 // degree, largest degree first) with the per-degree launch shapes
 // block[d], cps[d], lanes per polynomial lanes[d] and polish warps pw[d]
 // (> 0: the warp-specialised form, mixed mode, degrees up to 8; UNEVEN_SPLIT:
-// the split-register form, FP64 polish, degrees 4 to 12).
+// the split-register form, degrees 4 to 12, compensated polish 7 to 11).
 template <typename In, int MODE>
 int launch_uneven_bins(const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets, const int *block,
                        const int *cps, const int *lanes, const int *pw, bool fork, cudaStream_t st);

@@ -150,7 +150,7 @@ template <int N, typename In, int MODE>
 static int launch_degree_bin(const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets, int block,
                              int ctas_per_sm, int lanes, int polish_warps, cudaStream_t st)
 {
-    if constexpr (MODE == MODE_MIXED_FP64) {
+    if constexpr (MODE != MODE_PLAIN) {
         if (polish_warps == UNEVEN_SPLIT)
             return launch_uneven_split(N, std::is_same<In, float2>::value ? RD_C64 : RD_C128, a, L, offsets, st);
     }

@@ -6,7 +6,7 @@ namespace rd {
 
 int launch_uneven_split_c128(int degree, const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets, cudaStream_t st)
 {
-    return launch_uneven_split_degree<double2>(degree, a, L, offsets, st);
+    return launch_uneven_split_degree<double2, MODE_MIXED_FP64>(degree, a, L, offsets, st);
 }
 
 }  // namespace rd
