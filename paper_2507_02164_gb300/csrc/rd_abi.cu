@@ -33,6 +33,7 @@ int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const
                   const int *pw, bool fork, const bool *open_shape, cudaStream_t st);
 bool group_takes(int degree, int64_t n, bool mixed);
 int launch_group(int degree, rd_dtype dt, bool mixed, const SolveArgs &a, cudaStream_t st);
+int launch_pool(int degree, rd_dtype dt, const SolveArgs &a, cudaStream_t st);
 int launch_solve_split(int degree, rd_dtype dt, const SolveArgs &a, cudaStream_t st);
 int launch_l2(const double *samples, int64_t n, int nr, int degree, double *coeffs, int precision,
               cudaStream_t st);
@@ -169,9 +170,23 @@ bool split_takes(int degree, rd_dtype dtype, int64_t n, bool mixed, int polish_m
     return per_sm >= (degree <= 6 ? 576 : (degree <= 8 ? 352 : 224));
 }
 
+// FP64 sweeps of enough polynomials take the pool solver (rd_pool.cu): fewer
+// leave its pools too small to keep the lanes busy. Measured (us, complex128),
+// pool against one warp per CTA of the one-role kernel, by polynomials per SM:
+//   degree      192          256          320          448          640          1024         2304
+//    3       111 / 96    126 / 121    158 / 154    205 / 211    269 / 296    422 / 457    948 / 1013
+//    4       288 / 267   320 / 331    378 / 417    495 / 561    671 / 785   1058 / 1270  2332 / 2682
+//    5       357 / 356   428 / 442    526 / 556    707 / 837    967 / 1178  1548 / 1762  3426 / 3695
+//    6       655 / 630   788 / 827    950 / 1206  1272 / 1418  1828 / 2023  2806 / 3084  6269 / 6823
+//    7       765 / 761   945 / 956   1159 / 1383  1649 / 1683  2277 / 2428  3618 / 3658  7929 / 8123
+bool pool_takes(int degree, int64_t n)
+{
+    return degree >= 3 && degree <= 7 && n / rd_sm_count_cached() >= (degree == 3 ? 448 : 256);
+}
+
 // The launch shape of any other uniform batch, when the caller left it open: one
-// warp per CTA, which spreads a ragged wave over all SMs. Plain degree 6 65,536
-// 1164 us against 1285 with 128 threads, degree 12 20,000 2359 against 3339; mixed
+// warp per CTA, which spreads a ragged wave over all SMs. Plain degree 6 20,000
+// 571 us against 777 with 128 threads, degree 12 20,000 2359 against 3339; mixed
 // degree 12 20,000 198 against 227; compensated 7 150,000 193 against 207 (128) and
 // 223 (256); equal on full waves. Except the compensated polish of degrees 5 and 6,
 // 256 threads (warps that start together share the instruction cache): degree 6
@@ -266,6 +281,7 @@ int solve_common(const void *coeffs, rd_dtype dtype, int degree, int64_t n, rd_m
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (shape_open(p)) {
         if (rd::group_takes(degree, n, mode == RD_MIXED)) return rd::launch_group(degree, dtype, mode == RD_MIXED, a, st);
+        if (mode != RD_MIXED && pool_takes(degree, n)) return rd::launch_pool(degree, dtype, a, st);
         if (split_takes(degree, dtype, n, mode == RD_MIXED, p.polish_mode)) return rd::launch_solve_split(degree, dtype, a, st);
         open_shape(p, degree, n, mode == RD_MIXED);
     }
