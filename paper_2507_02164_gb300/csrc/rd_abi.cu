@@ -186,15 +186,26 @@ bool pool_takes(int degree, int64_t n)
 
 // The launch shape of any other uniform batch, when the caller left it open: one
 // warp per CTA, which spreads a ragged wave over all SMs. Plain degree 6 20,000
-// 571 us against 777 with 128 threads, degree 12 20,000 2359 against 3339; mixed
-// degree 12 20,000 198 against 227; compensated 7 150,000 193 against 207 (128) and
-// 223 (256); equal on full waves. Except the compensated polish of degrees 5 and 6,
-// 256 threads (warps that start together share the instruction cache): degree 6
-// 300,000 265 against 278, 2^20 904 against 973, 2^19 448 against 470.
+// 571 us against 777 with 128 threads, 7858 343 against 362; mixed degree 12 20,000
+// 198 against 227; compensated 7 150,000 193 against 207 (128) and 223 (256); equal
+// on full waves. Two exceptions:
+//   one wave of 128-thread CTAs: their four warps have a sub-partition each and
+//     share the instruction cache (32 / 128 threads): mixed 7858 degree 12 191 /
+//     181; 18,000 12 191 / 185, plain 6 408 / 382, 12 2258 / 2112. (Plain batches of
+//     at most three warps per SM want the spread: degree 12 4000 1890 / 1971.) The
+//     compensated polish, which does not live on the FP64 unit, up to two warps
+//     per sub-partition (8 complex128 30,000 90 / 86), degree 12 always (100,003
+//     543 / 534, 300,007 1462 / 1422).
+//   compensated polish, degrees 5 and 6, many waves: 256 threads: degree 6 300,000
+//     265 against 278, 2^20 904 against 973, 2^19 448 against 470.
 void open_shape(rd_params &p, int degree, int64_t n, bool mixed)
 {
+    const int64_t sms = rd_sm_count_cached();
     const bool df = mixed && p.polish_mode == RD_POLISH_DF;
-    p.block = df && (degree == 5 || degree == 6) && n / rd_sm_count_cached() >= 1536 ? 256 : 32;
+    p.block = 32;
+    if (n <= (df ? 256 : 128) * sms && (mixed || n > 96 * sms)) p.block = 128;
+    if (df && degree == 12) p.block = 128;
+    if (df && (degree == 5 || degree == 6) && n >= 1536 * sms) p.block = 256;
 }
 
 // Validate a tile clip (host struct, device arrays) for n polynomials.
