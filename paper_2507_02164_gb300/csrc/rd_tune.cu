@@ -123,8 +123,9 @@ struct Shape {
 // The candidates: one-role shapes (lanes 1, and 2 from degree 2; 32..256
 // threads; the occupancy maximum or fewer CTAs per SM), then for RD_MIXED the
 // warp-specialised shapes: up to 16 warps per CTA at degrees <= 6 (about 128
-// registers), up to 8 above (255). A polish warp keeps about one FP64
-// instruction in flight, so the FP64 pipe wants about ten polish warps per SM.
+// registers), up to 8 above (255). Each SM sub-partition has an FP64 unit, which
+// idles while none of its warps is in FP64 work: with one register count for
+// both roles about ten polish warps of sixteen keep it busiest.
 std::vector<Shape> candidates(int degree, rd_mode mode, int polish_mode)
 {
     std::vector<Shape> v;
@@ -138,9 +139,9 @@ std::vector<Shape> candidates(int degree, rd_mode mode, int polish_mode)
             for (int k = 0; k < 3; ++k) v.push_back({lanes, b, cps[k], 0});
         }
     if (mode == RD_MIXED) {
-        // the FP64 polish wants about ten polish warps (one FP64 instruction in
-        // flight per warp); the compensated polish is FP32 work of about the
-        // sweeps' size and wants an even split
+        // the FP64 polish wants two to three polish warps in each sub-partition; the
+        // compensated polish is FP32 work of about the sweeps' size and wants an
+        // even split
         static const int ws_small[][2] = {{512, 8}, {512, 9}, {512, 10}, {512, 11}, {256, 4}, {256, 5}, {192, 3}, {192, 4}};
         static const int ws_large[][2] = {{96, 1}, {96, 2}, {128, 1}, {128, 2}, {192, 2}, {192, 3}, {192, 4},
                                           {256, 3}, {256, 4}};

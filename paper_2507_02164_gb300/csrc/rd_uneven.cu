@@ -10,10 +10,11 @@
 // Workspace (caller-allocated, contents overwritten, 256-byte aligned):
 //   [header 512 B][perm: uint32 per polynomial][bins: the coefficients again,
 //   coefficient-major within each degree bin]
-// Launch sequence on the caller's stream (graph-capturable, no allocation,
-// no synchronisation): clear header -> count -> scan -> pack -> one
-// persistent solve kernel per degree, largest degree first, each with its
-// own register allocation and its own task queue.
+// Launch sequence (graph-capturable, no allocation, no synchronisation): clear
+// header -> count, then for small batches one kernel that gives every polynomial
+// a group of lanes (rd_group.cu), else scan -> pack -> one persistent solve kernel
+// per degree, largest degree first, each with its own register allocation and
+// its own task queue, on several chains of streams (rd_uneven_bins.cuh).
 #include "rd_uneven.cuh"
 
 namespace rd {
@@ -265,7 +266,7 @@ size_t uneven_workspace_bytes(int64_t n, int64_t n_coeffs, rd_dtype dt)
 // Whether the degree bins 4 to 12 (compensated polish 7 to 11) take the split-register solver
 // (rd_solve_split.cuh) where the caller left their launch shapes open. The
 // bins' sizes exist only on the device, so the line is drawn on n; each split
-// kernel takes whole SMs, so small bins lose the overlap of the two chains.
+// kernel takes whole SMs, so small bins lose the overlap of the chains.
 // Measured (us, degrees 2..12, complex64, split / one role): 300,000 1030 / 930,
 // 2^19 1560 / 1430, 2^20 2385 / 2498, 2^22 7909 / 9357 (complex128 2574 / 2621,
 // 8702 / 9864). Compensated polish: 2^20 1932 / 1888, 1,500,000 2583 / 2658,
