@@ -174,11 +174,12 @@ bool split_takes(int degree, rd_dtype dtype, int64_t n, bool mixed, int polish_m
 // leave its pools too small to keep the lanes busy. Measured (us, complex128),
 // pool against one warp per CTA of the one-role kernel, by polynomials per SM:
 //   degree      192          256          320          448          640          1024         2304
-//    3       111 / 96    126 / 121    158 / 154    205 / 211    269 / 296    422 / 457    948 / 1013
-//    4       288 / 267   320 / 331    378 / 417    495 / 561    671 / 785   1058 / 1270  2332 / 2682
-//    5       357 / 356   428 / 442    526 / 556    707 / 837    967 / 1178  1548 / 1762  3426 / 3695
-//    6       655 / 630   788 / 827    950 / 1206  1272 / 1418  1828 / 2023  2806 / 3084  6269 / 6823
-//    7       765 / 761   945 / 956   1159 / 1383  1649 / 1683  2277 / 2428  3618 / 3658  7929 / 8123
+//    3       111 / 96    126 / 121    158 / 154    199 / 212    275 / 296    386 / 456    849 / 1012
+//    4       288 / 267   320 / 331    378 / 417    501 / 561    662 / 783    976 / 1269  2215 / 2678
+//    5       357 / 356   428 / 443    526 / 556    694 / 836    944 / 1177  1498 / 1759  3330 / 3696
+//    6       655 / 630   788 / 827    949 / 1204  1235 / 1416  1827 / 2020  2724 / 3080  6129 / 6811
+//    7       765 / 761   944 / 956   1158 / 1382  1649 / 1681  2276 / 2426  3613 / 3654  7696 / 8120
+// 2^22 Littlewood polynomials of degree 6, complex64: 61.1 against 63.1 ms.
 bool pool_takes(int degree, int64_t n)
 {
     return degree >= 3 && degree <= 7 && n / rd_sm_count_cached() >= (degree == 3 ? 448 : 256);

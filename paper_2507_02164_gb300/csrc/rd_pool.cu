@@ -9,26 +9,26 @@
 // sweep, and 65,536 polynomials are 3.4 warps per sub-partition, the time of
 // four. Beside that, moving a matrix is free: a sweep of a 6 x 6 block takes
 // some 50,000 cycles, its load from and store to shared memory about 500.
-// So there is one warp per sub-partition, with an equal share of the batch in
-// shared memory (up to 135 polynomials of degree 6), and before each sweep it
-// takes the 32 largest active blocks. Simulated for degree 6 and a pool of 108:
+// So there is one warp per sub-partition (two where the batch fills their pools,
+// launch_pool_n), with an equal share of the batch in shared memory (up to 135
+// polynomials of degree 6), and before each sweep it takes the 32 largest active
+// blocks. Simulated for degree 6 and a pool of 108:
 // 18.4 warp sweeps per 32 polynomials instead of 21.5 (mean of a polynomial:
 // 16.8), and 0.85 of the FP64 instructions. Every polynomial takes the same
 // steps in the same order as in sweep_lane: the same bits and counters.
 // Measured (us, degree 6, complex128, roots drawn from the disk): 65,536 1468 ->
-// 1238, 40,000 1171 -> 817, 350,208 6823 -> 6269. Two warps per sub-partition
-// with a pool each: 1218, but 948 and 6400; sharing one pool by compare-and-swap:
-// 1202, 922, 6380; eight warps on one pool per SM: 1248, 1006: all within the
-// FP64 time of the sweeps that they save or add.
+// 1218, 40,000 1171 -> 817, 2^18 5168 -> 4676. Two warps that share one pool by
+// compare-and-swap: 1202, 922, 4716; eight on one pool per SM: 1248, 1006, 4703:
+// within the FP64 time of the sweeps that they save or add.
 #include "rd_solve.cuh"
 
 namespace rd {
 
-template <int N>
+template <int N, int W>
 struct Pool {
     static constexpr int ENTRIES = N * (N + 1) / 2 + N - 1;  // of an upper Hessenberg matrix
     static constexpr int SLOT_BYTES = 16 * ENTRIES + 8;
-    static constexpr int WARPS = 4;                          // one in each sub-partition of an SM
+    static constexpr int WARPS = W;                          // of a CTA, one CTA per SM
     static constexpr int FIT = 225 * 1024 / WARPS / SLOT_BYTES;
     static constexpr int SLOTS = FIT < 160 ? FIT : 160;
 };
@@ -52,20 +52,20 @@ __device__ __forceinline__ void pool_deflate(const SolveArgs &A, const cx<double
     }
 }
 
-template <int N, typename In>
-__global__ void __launch_bounds__(32 * Pool<N>::WARPS, 1) pool_kernel(SolveArgs A, int slots, int rounds)
+template <int N, int W, typename In>
+__global__ void __launch_bounds__(32 * W, 1) pool_kernel(SolveArgs A, int slots, int rounds)
 {
     extern __shared__ __align__(16) double2 pool_smem[];
     __shared__ unsigned long long acc[ST_WORDS];
-    __shared__ int lists[Pool<N>::WARPS][32];
+    __shared__ int lists[Pool<N, W>::WARPS][32];
     const CtaStats S = stats_begin(acc, A.stats);
     const UniformMap map{{}, A.n};
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double2 *ent = pool_smem + (size_t)warp * Pool<N>::ENTRIES * slots;  // entry e of slot p at e * slots + p
-    int *state = reinterpret_cast<int *>(pool_smem + (size_t)Pool<N>::WARPS * Pool<N>::ENTRIES * slots) + warp * 2 * slots;
+    double2 *ent = pool_smem + (size_t)warp * Pool<N, W>::ENTRIES * slots;  // entry e of slot p at e * slots + p
+    int *state = reinterpret_cast<int *>(pool_smem + (size_t)Pool<N, W>::WARPS * Pool<N, W>::ENTRIES * slots) + warp * 2 * slots;
     int *sweeps_made = state + slots;
     int *list = lists[warp];
-    const int64_t warps = (int64_t)gridDim.x * Pool<N>::WARPS, w = blockIdx.x + (int64_t)gridDim.x * warp;
+    const int64_t warps = (int64_t)gridDim.x * Pool<N, W>::WARPS, w = blockIdx.x + (int64_t)gridDim.x * warp;
 
     auto put = [&](const cx<double> (&h)[N][N], int p, int m, int its, int flags) {
         int e = 0;
@@ -173,19 +173,39 @@ __global__ void __launch_bounds__(32 * Pool<N>::WARPS, 1) pool_kernel(SolveArgs 
     stats_end(S, A.stats);
 }
 
+// A batch of n in equal shares: as many rounds as the slots ask for.
+template <int N, int W>
+static void pool_shares(int64_t n, int64_t &rounds, int64_t &slots)
+{
+    const int64_t warps = (int64_t)rd_sm_count_cached() * W, most = Pool<N, W>::SLOTS;
+    rounds = (n + warps * most - 1) / (warps * most);
+    slots = (n + warps * rounds - 1) / (warps * rounds);
+}
+
+template <int N, int W, typename In>
+static int launch_pool_warps(const SolveArgs &a, cudaStream_t st)
+{
+    using C = Pool<N, W>;
+    int64_t rounds, slots;
+    pool_shares<N, W>(a.n, rounds, slots);
+    auto kern = pool_kernel<N, W, In>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, W * C::SLOT_BYTES * C::SLOTS) != cudaSuccess)
+        return rd_check_launch("cudaFuncSetAttribute(pool_kernel)");
+    kern<<<(unsigned)rd_sm_count_cached(), 32 * W, (size_t)(W * C::SLOT_BYTES * slots), st>>>(a, (int)slots, (int)rounds);
+    return rd_check_launch("pool_kernel");
+}
+
+// Two warps per sub-partition hide what a lone one waits for (selection, matrix
+// moves, square roots) but halve the pools: taken where a pool still holds one and
+// a half warps' worth. Measured (us, complex128, one / two): 42 to 43 slots degree
+// 6 100,003 1911 / 2108, 7 2348 / 2353; 54 slots 6 65,536 1238 / 1218, 2^18 4732 /
+// 4676; 80 and more 3 2^18 713 / 666, 4 100,003 614 / 564, 5 100,003 1041 / 953.
 template <int N, typename In>
 static int launch_pool_n(const SolveArgs &a, cudaStream_t st)
 {
-    using C = Pool<N>;
-    const int64_t sms = rd_sm_count_cached(), warps = sms * C::WARPS;
-    // as many rounds as the slots ask for, and then equal ones
-    const int64_t rounds = (a.n + warps * C::SLOTS - 1) / (warps * C::SLOTS);
-    const int slots = (int)((a.n + warps * rounds - 1) / (warps * rounds));
-    auto kern = pool_kernel<N, In>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::WARPS * C::SLOT_BYTES * C::SLOTS) != cudaSuccess)
-        return rd_check_launch("cudaFuncSetAttribute(pool_kernel)");
-    kern<<<(unsigned)sms, 32 * C::WARPS, (size_t)C::WARPS * C::SLOT_BYTES * slots, st>>>(a, slots, (int)rounds);
-    return rd_check_launch("pool_kernel");
+    int64_t rounds, slots;
+    pool_shares<N, 8>(a.n, rounds, slots);
+    return slots >= 48 ? launch_pool_warps<N, 8, In>(a, st) : launch_pool_warps<N, 4, In>(a, st);
 }
 
 // Degree 8 (83 polynomials fit, the sweep spills) gains less than it loses at
