@@ -46,9 +46,9 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-# Units that instantiate the register-resident solver for many degrees take
+# Units that instantiate a solver for many degrees take
 # 10-25 s each, the rest 1-9 s: start them first so the pool ends together.
-HEAVY = ("rd_solve", "rd_uneven_bins", "rd_backward")
+HEAVY = ("rd_solve", "rd_uneven_bins", "rd_uneven_split", "rd_backward", "rd_pool", "rd_group")
 
 
 def _compile_order(srcs):
