@@ -161,11 +161,12 @@ bool shape_open(const rd_params &p)
 //   10           176 / 187  204 / 213  265 / 297  296 / 339  392 / 458  754 / 929  1286 / 1621
 //   11           226 / 246  268 / 261  349 / 374  396 / 394  526 / 546  997 / 1101 1672 / 1911
 // (25,000: 9 100 / 92, 11 141 / 138).
-bool split_takes(int degree, rd_dtype dtype, int64_t n, bool mixed, int polish_mode)
+// (Only with sweep bounds that its waits allow for: split_waits_ok.)
+bool split_takes(int degree, rd_dtype dtype, int64_t n, bool mixed, const rd_params &p)
 {
-    if (!mixed || degree < 4) return false;
+    if (!mixed || degree < 4 || !rd::split_waits_ok(degree, p.max_iters, p.fixed_sweeps)) return false;
     const int64_t per_sm = n / rd_sm_count_cached();
-    if (polish_mode == RD_POLISH_DF) return degree >= 7 && degree <= 11 && per_sm >= (degree == 7 ? 1536 : (degree == 8 ? 640 : 256));
+    if (p.polish_mode == RD_POLISH_DF) return degree >= 7 && degree <= 11 && per_sm >= (degree == 7 ? 1536 : (degree == 8 ? 640 : 256));
     if (degree == 4) return dtype == RD_C64 && per_sm >= 640;
     return per_sm >= (degree <= 6 ? 576 : (degree <= 8 ? 352 : 224));
 }
@@ -294,7 +295,7 @@ int solve_common(const void *coeffs, rd_dtype dtype, int degree, int64_t n, rd_m
     if (shape_open(p)) {
         if (rd::group_takes(degree, n, mode == RD_MIXED)) return rd::launch_group(degree, dtype, mode == RD_MIXED, a, st);
         if (mode != RD_MIXED && pool_takes(degree, n)) return rd::launch_pool(degree, dtype, a, st);
-        if (split_takes(degree, dtype, n, mode == RD_MIXED, p.polish_mode)) return rd::launch_solve_split(degree, dtype, a, st);
+        if (split_takes(degree, dtype, n, mode == RD_MIXED, p)) return rd::launch_solve_split(degree, dtype, a, st);
         open_shape(p, degree, n, mode == RD_MIXED);
     }
     if (p.polish_warps > 0) {

@@ -306,7 +306,10 @@ int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const
     int bins_pw[16];
     const bool split = uneven_split_takes(n, mixed, a.polish_mode), df = a.polish_mode == RD_POLISH_DF;
     const int first = df ? 7 : 4, last = df ? 11 : UNEVEN_MAX_DEG;
-    for (int d = 0; d < 16; ++d) bins_pw[d] = split && open_shape[d] && d >= first && d <= last ? UNEVEN_SPLIT : pw[d];
+    for (int d = 0; d < 16; ++d) {
+        const bool takes = split && open_shape[d] && d >= first && d <= last && split_waits_ok(d, a.max_iters, a.fixed_sweeps);
+        bins_pw[d] = takes ? UNEVEN_SPLIT : pw[d];
+    }
     pw = bins_pw;
     uneven_scan_kernel<<<1, 32, 0, st>>>(L.hdr, n_coeffs);
     if ((rc = rd_check_launch("uneven_scan_kernel"))) return rc;

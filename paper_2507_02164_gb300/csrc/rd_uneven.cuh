@@ -104,6 +104,17 @@ struct UnevenFork {
 int uneven_fork(cudaStream_t st, int sides, UnevenFork *out, bool retry = false);
 int uneven_join(cudaStream_t st, const UnevenFork &f);
 
+// The split-register solver hands tasks of 32 polynomials between warps with
+// waits that give up after 2 s (WS_WAIT_NS). A warp waits for about three
+// tasks at most, and a sweep takes 3 us (degree 12, 1.1e6 sweeps per polynomial
+// in 3.4 s), at the largest block less than 10, so at most 4,096 sweeps per
+// polynomial (the defaults: 440 at degree 12) keep every wait below 0.15 s. A
+// call that allows more takes the forms that wait for nothing.
+inline bool split_waits_ok(int degree, int max_iters, int fixed_sweeps)
+{
+    return (int64_t)(degree - 1) * (fixed_sweeps > 0 ? fixed_sweeps : max_iters) <= 4096;
+}
+
 // Large bins: the split-register solver (rd_solve_split.cuh).
 int launch_uneven_split(int degree, rd_dtype dt, const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets,
                         cudaStream_t st);
