@@ -9,6 +9,7 @@
 
 #include "rd_common.cuh"
 #include "rd_solve.cuh"
+#include "rd_uneven.cuh"
 
 namespace rd {
 int launch_solve_mixed(int degree, rd_dtype dt, const SolveArgs &a, int block, int ctas_per_sm, cudaStream_t st);
