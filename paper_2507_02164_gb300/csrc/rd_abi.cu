@@ -296,7 +296,10 @@ int solve_common(const void *coeffs, rd_dtype dtype, int degree, int64_t n, rd_m
     if (shape_open(p)) {
         if (rd::group_takes(degree, n, mode == RD_MIXED)) return rd::launch_group(degree, dtype, mode == RD_MIXED, a, st);
         if (mode != RD_MIXED && pool_takes(degree, n)) return rd::launch_pool(degree, dtype, a, st);
-        if (split_takes(degree, dtype, n, mode == RD_MIXED, p)) return rd::launch_solve_split(degree, dtype, a, st);
+        if (split_takes(degree, dtype, n, mode == RD_MIXED, p)) {
+            rc = rd::launch_solve_split(degree, dtype, a, st);
+            if (rc != rd::SPLIT_DECLINED) return rc;
+        }
         open_shape(p, degree, n, mode == RD_MIXED);
     }
     if (p.polish_warps > 0) {

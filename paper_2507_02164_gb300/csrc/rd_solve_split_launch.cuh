@@ -8,22 +8,25 @@
 
 namespace rd {
 
-// Once per kernel and device: the shared-memory opt-in, and the check that
-// the kernel was built with the registers per thread that its roles' shares
-// were added up against (a share above what the launch holds would wait
-// forever). Host calls outside any stream order, so a capture may follow.
+// Once per kernel and device: the check that the kernel was built with the
+// registers per thread that its roles' shares were added up against (a share
+// above what the launch holds would wait forever), and the shared-memory
+// opt-in. With another count SPLIT_DECLINED: the caller takes the one-role
+// kernel. Host calls outside any stream order, so a capture may follow.
 template <int N, typename In, int MODE, typename Kern>
 static int split_ready(Kern kern, std::atomic<int> (&ready)[64])
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return rd_check_launch("cudaGetDevice");
     if (dev < 0 || dev >= 64) return rd_set_error(RD_EUNSUPPORTED, "device %d: at most 64 devices", dev);
-    if (ready[dev].load()) return RD_OK;
+    const int known = ready[dev].load();
+    if (known) return known > 0 ? RD_OK : SPLIT_DECLINED;
     cudaFuncAttributes attr;
     if (cudaFuncGetAttributes(&attr, kern) != cudaSuccess) return rd_check_launch("cudaFuncGetAttributes(split kernel)");
-    if (attr.numRegs != Split<N, MODE>::LAUNCH_REGS)
-        return rd_set_error(RD_EUNSUPPORTED, "split kernel of degree %d built with %d registers per thread, %d expected", N,
-                            attr.numRegs, Split<N, MODE>::LAUNCH_REGS);
+    if (attr.numRegs != Split<N, MODE>::LAUNCH_REGS) {
+        ready[dev].store(-1);
+        return SPLIT_DECLINED;
+    }
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_smem_bytes<N, In, MODE>()) != cudaSuccess)
         return rd_check_launch("cudaFuncSetAttribute(split kernel)");
     ready[dev].store(1);

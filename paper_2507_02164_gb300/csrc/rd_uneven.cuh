@@ -119,6 +119,7 @@ inline bool split_waits_ok(int degree, int max_iters, int fixed_sweeps)
 int launch_uneven_split(int degree, rd_dtype dt, const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets,
                         cudaStream_t st);
 constexpr int UNEVEN_SPLIT = -1;  // in launch_uneven_bins' pw[d]
+constexpr int SPLIT_DECLINED = 1;  // launch_solve_split, launch_uneven_split: nothing enqueued, take the one-role kernel
 
 // Small batches: every polynomial by a group of lanes, no bins (rd_group.cu).
 int launch_uneven_group(const SolveArgs &a, rd_dtype dt, const UnevenArgs &U, const UnevenHeader *hdr, bool mixed,

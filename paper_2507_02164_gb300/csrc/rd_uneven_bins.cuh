@@ -151,8 +151,10 @@ static int launch_degree_bin(const SolveArgs &a, const UnevenLayout &L, const in
                              int ctas_per_sm, int lanes, int polish_warps, cudaStream_t st)
 {
     if constexpr (MODE != MODE_PLAIN) {
-        if (polish_warps == UNEVEN_SPLIT)
-            return launch_uneven_split(N, std::is_same<In, float2>::value ? RD_C64 : RD_C128, a, L, offsets, st);
+        if (polish_warps == UNEVEN_SPLIT) {
+            const int rc = launch_uneven_split(N, std::is_same<In, float2>::value ? RD_C64 : RD_C128, a, L, offsets, st);
+            if (rc != SPLIT_DECLINED) return rc;
+        }
     }
     if constexpr (MODE != MODE_PLAIN && N <= UNEVEN_WS_MAX_DEG) {
         if (polish_warps > 0) return launch_uneven_ws<N, In, MODE>(a, L, offsets, block, polish_warps, st);
