@@ -232,9 +232,11 @@ int uneven_fork(cudaStream_t st, int sides, UnevenFork *out, bool retry)
     e = cudaEventRecord(f.fork, st);
     for (int k = 0; k < sides && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(f.side[k], f.fork, 0);
     if (e != cudaSuccess) {
-        // handles made before a cudaDeviceReset are gone: forget them (they
-        // cannot be destroyed any more) and make new ones, once
-        if (e != cudaErrorInvalidResourceHandle || retry) return rd_set_error(RD_ECUDA, "uneven fork: %s", cudaGetErrorString(e));
+        // handles made before a cudaDeviceReset are gone (the runtime answers with
+        // either code): forget them (they cannot be destroyed any more) and make
+        // new ones, once
+        if ((e != cudaErrorInvalidResourceHandle && e != cudaErrorContextIsDestroyed) || retry)
+            return rd_set_error(RD_ECUDA, "uneven fork: %s", cudaGetErrorString(e));
         cudaGetLastError();
         f.forget();
         return uneven_fork(st, sides, out, true);
@@ -294,12 +296,12 @@ int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const
     bool all_open = true;
     for (int d = 1; d <= UNEVEN_MAX_DEG; ++d) all_open &= open_shape[d];
     if (all_open && uneven_group_takes(n, mixed)) {
-        // the first call of a host thread makes the helper streams whatever its
-        // size, so that a larger batch can be captured after it
+        // the first call of a host thread, or after a device reset, makes the helper
+        // streams whatever its size, so that a larger batch can be captured after it
         cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
         if (fork && cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) {
-            ForkState *state = nullptr;
-            if ((rc = uneven_handles(&state))) return rc;
+            UnevenFork none;
+            if ((rc = uneven_fork(st, 0, &none))) return rc;
         }
         return launch_uneven_group(a, dt, U, L.hdr, mixed, st);
     }
