@@ -427,6 +427,13 @@ struct CtaStats {
         unsigned w = __reduce_add_sync(0xffffffffu, v);
         if ((threadIdx.x & 31) == 0 && w) atomicAdd(acc + k, (unsigned long long)w);
     }
+    // The same where the warp's sum may exceed 32 bits: the halves apart.
+    __device__ void add_wide(int k, unsigned v) const
+    {
+        if (!acc) return;
+        const unsigned lo = __reduce_add_sync(0xffffffffu, v & 0xffffu), hi = __reduce_add_sync(0xffffffffu, v >> 16);
+        if ((threadIdx.x & 31) == 0) atomicAdd(acc + k, ((unsigned long long)hi << 16) + lo);
+    }
 };
 
 // Zero the CTA's counters (all threads of the CTA call this).

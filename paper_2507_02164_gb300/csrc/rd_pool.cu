@@ -149,10 +149,12 @@ __global__ void __launch_bounds__(32 * W, 1) pool_kernel(SolveArgs A, int slots,
             }
             __syncwarp();
         }
-        S.add(ST_SWEEPS, n_sweeps);
-        S.add(ST_PAIRS, n_pairs);
-        S.add(ST_ROTS, n_rots);
-        S.add(ST_F64, 20u * n_pairs + 24u * n_rots + 60u * n_sweeps);
+        // A lane's own sums of a round fit 32 bits (at most 100,000 sweeps per
+        // eigenvalue: 3.3e9 flops at degree 7), a pool's do not
+        S.add_wide(ST_SWEEPS, n_sweeps);
+        S.add_wide(ST_PAIRS, n_pairs);
+        S.add_wide(ST_ROTS, n_rots);
+        S.add_wide(ST_F64, 20u * n_pairs + 24u * n_rots + 60u * n_sweeps);
         // ---- the roots: the diagonals
         for (int q = 0; q < count; q += 32) {
             const int p = q + lane;
