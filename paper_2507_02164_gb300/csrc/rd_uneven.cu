@@ -293,9 +293,14 @@ int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const
     if (ctas < 1) ctas = 1;
     uneven_count_kernel<<<(unsigned)ctas, tb, 0, st>>>(U, L.hdr, a.roots, a.status, a.stats);
     if ((rc = rd_check_launch("uneven_count_kernel"))) return rc;
+    // Roots that go over the coefficients: the bins read their own copy, the group
+    // kernel would read the caller's array while other polynomials' roots are stored
+    const int64_t n_roots = n_coeffs > n ? n_coeffs - n : 0;
+    const uintptr_t c0 = reinterpret_cast<uintptr_t>(a.coeffs), r0 = reinterpret_cast<uintptr_t>(a.roots);
+    const bool in_place = r0 && r0 < c0 + (uint64_t)n_coeffs * (dt == RD_C64 ? 8 : 16) && c0 < r0 + (uint64_t)n_roots * 16;
     bool all_open = true;
     for (int d = 1; d <= UNEVEN_MAX_DEG; ++d) all_open &= open_shape[d];
-    if (all_open && uneven_group_takes(n, mixed)) {
+    if (all_open && !in_place && uneven_group_takes(n, mixed)) {
         // the first call of a host thread, or after a device reset, makes the helper
         // streams whatever its size, so that a larger batch can be captured after it
         cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
