@@ -607,7 +607,7 @@ __device__ __forceinline__ void finish_lane(const SolveArgs &A, const void *coef
                         const float az = sqrtf(norm2(zr));
                         good = residual_certain(N, moved, abs1(sub(zr, zf)), az, weight(az), abs1(af[N]), rtol);
                     }
-                    if (!__all_sync(0xffffffffu, good || degenerate)) {
+                    if (MODE == MODE_MIXED_DF || !__all_sync(0xffffffffu, good || degenerate)) {
                         cx<double> p = ad[N];
 #pragma unroll
                         for (int k = N - 1; k >= 0; --k) p = cfma(p, zj, ad[k]);
@@ -767,9 +767,17 @@ __device__ __forceinline__ void solve_warp(const SolveArgs &A, const void *coeff
 // against 1595), 10 and up lose (1084 against 1017).
 __host__ __device__ constexpr bool solve_twelve_warps(int n, int mode) { return mode != MODE_PLAIN && (n == 7 || n == 8); }
 
-// Uniform batch: warps stride over A.n polynomials, 32 at a time.
-template <int N, typename T, typename In, int MODE>
-__device__ __forceinline__ void solve_uniform(const SolveArgs &A)
+// Launch bounds of a one-role kernel: 256 threads with the registers that its
+// degree asks for, or (TWELVE) 384, which holds it to 168 registers.
+__host__ __device__ constexpr int solve_threads(bool twelve) { return twelve ? 384 : 256; }
+__host__ __device__ constexpr int solve_ctas(int n, int mode) { return (mode != MODE_PLAIN && n <= 6) ? 2 : 1; }
+
+// Uniform batch: warps stride over A.n polynomials, 32 at a time. (The body stays
+// in the kernel: called through a function that takes A by reference, the same
+// code spills 164 B instead of 8 to 28 at degree 11, complex128, and the
+// compensated polish is 5 % slower there, 2 to 8 % at degree 2.)
+template <int N, typename T, typename In, int MODE, bool TWELVE>
+__global__ void __launch_bounds__(solve_threads(TWELVE), solve_ctas(N, MODE)) solve_kernel(SolveArgs A)
 {
     const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int64_t warp_id = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -779,18 +787,6 @@ __device__ __forceinline__ void solve_uniform(const SolveArgs &A)
     for (int64_t base = warp_id * 32; base < A.n; base += warps_total * 32)
         solve_warp<N, T, In, MODE>(A, A.coeffs, A.n, base, map, S);
     stats_end(S, A.stats);
-}
-
-template <int N, typename T, typename In, int MODE>
-__global__ void __launch_bounds__(256, (MODE != MODE_PLAIN && N <= 6) ? 2 : 1) solve_kernel(SolveArgs A)
-{
-    solve_uniform<N, T, In, MODE>(A);
-}
-
-template <int N, typename T, typename In, int MODE>
-__global__ void __maxnreg__(168) solve_kernel_r168(SolveArgs A)
-{
-    solve_uniform<N, T, In, MODE>(A);
 }
 
 }  // namespace rd

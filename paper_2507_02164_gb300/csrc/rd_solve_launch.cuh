@@ -12,9 +12,9 @@ namespace rd {
 template <int N, typename T, typename In, int MODE>
 static auto solve_kernel_for(int64_t warps)
 {
-    auto kern = solve_kernel<N, T, In, MODE>;
+    auto kern = solve_kernel<N, T, In, MODE, false>;
     if constexpr (solve_twelve_warps(N, MODE))
-        if (warps > 8 * (int64_t)rd_sm_count_cached()) kern = solve_kernel_r168<N, T, In, MODE>;
+        if (warps > 8 * (int64_t)rd_sm_count_cached()) kern = solve_kernel<N, T, In, MODE, true>;
     return kern;
 }
 
