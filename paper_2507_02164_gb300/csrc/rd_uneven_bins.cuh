@@ -150,12 +150,17 @@ static int launch_degree_bin(const SolveArgs &a, const UnevenLayout &L, const in
             return launch_persistent(uneven_solve2_kernel<N, In, MODE>, a, L, offsets, block, ctas_per_sm, st,
                                      "uneven_solve2_kernel");
     }
-    if constexpr (solve_twelve_warps(N, MODE))
-        return launch_persistent(uneven_solve_kernel<N, In, MODE, true>, a, L, offsets, block, ctas_per_sm, st,
-                                 "uneven_solve_kernel");
-    else
-        return launch_persistent(uneven_solve_kernel<N, In, MODE, false>, a, L, offsets, block, ctas_per_sm, st,
-                                 "uneven_solve_kernel");
+    // At most eight warps per SM whatever the bin's share of the batch: free
+    // registers, as solve_kernel_for (us, all of degree 8, compensated, complex64,
+    // 168 / free: 17,000 124 / 107, 34,000 123 / 110, 50,000 130 / 165; FP64 polish
+    // 34,000 166 / 133, 50,000 167 / 210).
+    if constexpr (solve_twelve_warps(N, MODE)) {
+        if (a.n > 256 * (int64_t)rd_sm_count_cached())
+            return launch_persistent(uneven_solve_kernel<N, In, MODE, true>, a, L, offsets, block, ctas_per_sm, st,
+                                     "uneven_solve_kernel");
+    }
+    return launch_persistent(uneven_solve_kernel<N, In, MODE, false>, a, L, offsets, block, ctas_per_sm, st,
+                             "uneven_solve_kernel");
 }
 
 // The twelve degree bins run as parallel chains of persistent kernels, forked
