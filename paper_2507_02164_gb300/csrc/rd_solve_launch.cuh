@@ -7,14 +7,18 @@
 namespace rd {
 
 // Degrees 7 and 8 have a kernel held to 168 registers, for its twelve warps per
-// SM; a batch that has no more than eight takes the free one (compensated polish,
-// degree 8, complex128, 7858 polynomials: 70 us at 168 registers, 67 free).
+// SM instead of eight; it is the slower one per warp, and taken where it saves a
+// round of warps (us, degree 8, compensated, complex128, 168 / free: 7,858 70 /
+// 67; 52,781, 10.9 warps per SM, 113 / 138; 64,393, 13.2, 166 / 158; 78,559, 16.2,
+// 185 / 211).
 template <int N, typename T, typename In, int MODE>
 static auto solve_kernel_for(int64_t warps)
 {
     auto kern = solve_kernel<N, T, In, MODE, false>;
-    if constexpr (solve_twelve_warps(N, MODE))
-        if (warps > 8 * (int64_t)rd_sm_count_cached()) kern = solve_kernel<N, T, In, MODE, true>;
+    if constexpr (solve_twelve_warps(N, MODE)) {
+        const int64_t twelve = 12 * (int64_t)rd_sm_count_cached(), eight = 8 * (int64_t)rd_sm_count_cached();
+        if ((warps + twelve - 1) / twelve < (warps + eight - 1) / eight) kern = solve_kernel<N, T, In, MODE, true>;
+    }
     return kern;
 }
 
