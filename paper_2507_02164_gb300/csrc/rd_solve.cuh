@@ -772,12 +772,9 @@ __host__ __device__ constexpr bool solve_twelve_warps(int n, int mode) { return 
 __host__ __device__ constexpr int solve_threads(bool twelve) { return twelve ? 384 : 256; }
 __host__ __device__ constexpr int solve_ctas(int n, int mode) { return (mode != MODE_PLAIN && n <= 6) ? 2 : 1; }
 
-// Uniform batch: warps stride over A.n polynomials, 32 at a time. (The body stays
-// in the kernel: called through a function that takes A by reference, the same
-// code spills 164 B instead of 8 to 28 at degree 11, complex128, and the
-// compensated polish is 5 % slower there, 2 to 8 % at degree 2.)
-template <int N, typename T, typename In, int MODE, bool TWELVE>
-__global__ void __launch_bounds__(solve_threads(TWELVE), solve_ctas(N, MODE)) solve_kernel(SolveArgs A)
+// Uniform batch: warps stride over A.n polynomials, 32 at a time.
+template <int N, typename T, typename In, int MODE>
+__device__ __forceinline__ void solve_uniform(const SolveArgs &A)
 {
     const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int64_t warp_id = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -787,6 +784,30 @@ __global__ void __launch_bounds__(solve_threads(TWELVE), solve_ctas(N, MODE)) so
     for (int64_t base = warp_id * 32; base < A.n; base += warps_total * 32)
         solve_warp<N, T, In, MODE>(A, A.coeffs, A.n, base, map, S);
     stats_end(S, A.stats);
+}
+
+// The compiler allocates registers otherwise when the arguments are read in the
+// kernel itself instead of through a reference: degrees 1 and 2 are 2 to 9 %
+// faster for it and degree 11 of complex128 3 % (8 to 28 B of spills against
+// 164); degrees 3 to 6, 10 and 12 lose 1 to 2 %.
+template <int N, typename In, int MODE>
+constexpr bool solve_in_kernel = MODE != MODE_PLAIN && (N <= 2 || (N == 11 && std::is_same<In, double2>::value));
+
+template <int N, typename T, typename In, int MODE, bool TWELVE>
+__global__ void __launch_bounds__(solve_threads(TWELVE), solve_ctas(N, MODE)) solve_kernel(SolveArgs A)
+{
+    if constexpr (solve_in_kernel<N, In, MODE>) {
+        const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
+        const int64_t warp_id = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+        __shared__ unsigned long long acc[ST_WORDS];
+        const CtaStats S = stats_begin(acc, A.stats);
+        const UniformMap map{{}, A.n};
+        for (int64_t base = warp_id * 32; base < A.n; base += warps_total * 32)
+            solve_warp<N, T, In, MODE>(A, A.coeffs, A.n, base, map, S);
+        stats_end(S, A.stats);
+    } else {
+        solve_uniform<N, T, In, MODE>(A);
+    }
 }
 
 }  // namespace rd

@@ -16,9 +16,9 @@ namespace rd {
 // Persistent solver for the degree-N bin: each warp takes the next task of
 // the bin's queue (task = 32 consecutive slots) until the queue is empty.
 // One kernel per degree keeps each degree's own register allocation.
-template <int N, typename In, int MODE, bool TWELVE>
-__global__ void __launch_bounds__(solve_threads(TWELVE), solve_ctas(N, MODE))
-    uneven_solve_kernel(SolveArgs A, UnevenHeader *hdr, const uint32_t *perm, const char *bins, const int64_t *offsets)
+template <int N, typename In, int MODE>
+__device__ __forceinline__ void uneven_solve(const SolveArgs &A, UnevenHeader *hdr, const uint32_t *perm,
+                                             const char *bins, const int64_t *offsets)
 {
     using T = typename std::conditional<MODE != MODE_PLAIN, float, double>::type;
     __shared__ unsigned long long acc[ST_WORDS];
@@ -36,6 +36,13 @@ __global__ void __launch_bounds__(solve_threads(TWELVE), solve_ctas(N, MODE))
         solve_warp<N, T, In, MODE>(A, base, cnt, (int64_t)t * 32, map, S);
     }
     stats_end(S, A.stats);
+}
+
+template <int N, typename In, int MODE, bool TWELVE>
+__global__ void __launch_bounds__(solve_threads(TWELVE), solve_ctas(N, MODE))
+    uneven_solve_kernel(SolveArgs A, UnevenHeader *hdr, const uint32_t *perm, const char *bins, const int64_t *offsets)
+{
+    uneven_solve<N, In, MODE>(A, hdr, perm, bins, offsets);
 }
 
 // The same with two lanes per polynomial (rd_solve2.cuh): tasks of 16 slots.
