@@ -32,7 +32,7 @@ size_t uneven_workspace_bytes(int64_t n, int64_t n_coeffs, rd_dtype dt);
 int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const int64_t *offsets, int64_t n,
                   int64_t n_coeffs, bool mixed, void *ws, const int *block, const int *cps, const int *lanes,
                   const int *pw, bool fork, const bool *open_shape, cudaStream_t st);
-bool group_takes(int degree, int64_t n, bool mixed);
+bool group_takes(int degree, int64_t n, bool mixed, bool compensated);
 int launch_group(int degree, rd_dtype dt, bool mixed, const SolveArgs &a, cudaStream_t st);
 int launch_pool(int degree, rd_dtype dt, const SolveArgs &a, cudaStream_t st);
 int launch_solve_split(int degree, rd_dtype dt, const SolveArgs &a, cudaStream_t st);
@@ -294,7 +294,7 @@ int solve_common(const void *coeffs, rd_dtype dtype, int degree, int64_t n, rd_m
     if (n == 0) return RD_OK;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (shape_open(p)) {
-        if (rd::group_takes(degree, n, mode == RD_MIXED)) return rd::launch_group(degree, dtype, mode == RD_MIXED, a, st);
+        if (rd::group_takes(degree, n, mode == RD_MIXED, p.polish_mode == RD_POLISH_DF)) return rd::launch_group(degree, dtype, mode == RD_MIXED, a, st);
         if (mode != RD_MIXED && pool_takes(degree, n)) return rd::launch_pool(degree, dtype, a, st);
         if (split_takes(degree, dtype, n, mode == RD_MIXED, p)) {
             rc = rd::launch_solve_split(degree, dtype, a, st);

@@ -15,11 +15,14 @@ namespace rd {
 //             2432: degree 5  250 / 225    6  367 / 361    12  1847 / 1908
 // so the line lies at 40 polynomials per SM (mixed, from degree 3) and at 8
 // (plain, from degree 6: its FP64 instructions cost the same for one active
-// lane as for 32).
-bool group_takes(int degree, int64_t n, bool mixed)
+// lane as for 32). Degree 9, the first with 16 lanes per polynomial, has the least
+// to gain; with the compensated polish it ends earlier (complex64 4855 64.3 / 74.5,
+// 5923 79.4 / 74.4).
+bool group_takes(int degree, int64_t n, bool mixed, bool compensated)
 {
     const int64_t sms = rd_sm_count_cached();
-    return mixed ? degree >= 3 && n <= 40 * sms : degree >= 6 && n <= 8 * sms;
+    if (!mixed) return degree >= 6 && n <= 8 * sms;
+    return degree >= 3 && n <= (compensated && degree == 9 ? 36 : 40) * sms;
 }
 
 // The same for a packed batch of mixed degrees, which this solver takes in
