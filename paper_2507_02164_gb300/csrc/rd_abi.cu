@@ -190,8 +190,7 @@ bool pool_takes(int degree, int64_t n)
 // The launch shape of any other uniform batch, when the caller left it open: one
 // warp per CTA, which spreads a ragged wave over all SMs. Plain degree 6 20,000
 // 571 us against 777 with 128 threads, 7858 343 against 362; mixed degree 12 20,000
-// 198 against 227; compensated 7 150,000 193 against 207 (128) and 223 (256); equal
-// on full waves. Two exceptions:
+// 198 against 227; equal on full waves. Exceptions:
 //   one wave of 128-thread CTAs: their four warps have a sub-partition each and
 //     share the instruction cache (32 / 128 threads): mixed 7858 degree 12 191 /
 //     181; 18,000 12 191 / 185, plain 6 408 / 382, 12 2258 / 2112. (Plain batches of
@@ -199,14 +198,30 @@ bool pool_takes(int degree, int64_t n)
 //     compensated polish, which does not live on the FP64 unit, up to two warps
 //     per sub-partition (8 complex128 30,000 90 / 86), degree 12 always (100,003
 //     543 / 534, 300,007 1462 / 1422).
+//   up to twelve warps per SM, a batch that all but fills its CTAs of four or of
+//     two warps on every SM: single-warp CTAs then land unevenly on the
+//     sub-partitions (32 / 64 / 128 threads): 35,462, 7.3 warps, plain 12 3697 / 3505 /
+//     3501, plain 2 18.9 / 17.2 / 17.1; 29,067, 6.0, plain 9 (complex128) 1.13 / 1.00
+//     / 1.30 of the best; 52,781, 10.9, compensated 9 (complex128) 170 / 170 / 165.
+//   compensated polish, twelve to 32 warps per SM: two warps per CTA: 116,927
+//     degree 2 16.4 / 15.2 / 15.2, 78,559 degree 3 29.0 / 28.1 / 28.3.
 //   compensated polish, degrees 5 and 6, many waves: 256 threads: degree 6 300,000
 //     265 against 278, 2^20 904 against 973, 2^19 448 against 470.
 void open_shape(rd_params &p, int degree, int64_t n, bool mixed)
 {
-    const int64_t sms = rd_sm_count_cached();
+    const int64_t sms = rd_sm_count_cached(), per_sm = n / sms;
     const bool df = mixed && p.polish_mode == RD_POLISH_DF;
     p.block = 32;
-    if (n <= (df ? 256 : 128) * sms && (mixed || n > 96 * sms)) p.block = 128;
+    if (n <= (df ? 256 : 128) * sms) {
+        if (mixed || n > 96 * sms) p.block = 128;
+    } else if (n <= 384 * sms) {
+        if (per_sm % 128 == 0 || per_sm % 128 >= 88)
+            p.block = 128;
+        else if (!df && (per_sm % 64 == 0 || per_sm % 64 >= 56))
+            p.block = 64;
+    } else if (df && n <= 1024 * sms) {
+        p.block = 64;
+    }
     if (df && degree == 12) p.block = 128;
     if (df && (degree == 5 || degree == 6) && n >= 1536 * sms) p.block = 256;
 }
