@@ -336,22 +336,24 @@ struct CompHorner {
 
 // Split d * 2^-shift into hi + lo floats (|d * 2^-shift| <= 2): hi = d's
 // significand rounded to 24 bits, lo = the rest rounded to 24 bits (relative
-// error 2^-48). Magnitudes below the FP32 normal range become zero. On 32-bit
-// words: the low 29 significand bits are the remainder, less 2^29 where they
-// round hi up.
+// error 2^-48). Magnitudes below the FP32 normal range become zero.
 __device__ __forceinline__ dfl split_scaled(double d, int shift)
 {
-    const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
-    const unsigned sign = h & 0x80000000u;
-    const int E = (int)((h >> 20) & 0x7ffu);
-    const unsigned up = (l >> 28) & 1u;
-    const unsigned H = __funnelshift_l(l, (h & 0xfffffu) | 0x100000u, 3) + up;  // may be 2^24: the carry moves into the exponent
-    const int r = (int)(l & 0x1fffffffu) - (int)(up << 29);                     // |r| <= 2^28, exact remainder
-    const int e = E - 1023 - shift;                                             // unbiased exponent after scaling
-    const float hi = (e + 127 > 0 && E != 0) ? __uint_as_float(sign | (((unsigned)(e + 126) << 23) + H)) : 0.0f;
-    const int le = e - 52 + 127;
-    const float lo = (le > 0 && E != 0) ? __int2float_rn(r) * __uint_as_float(sign | ((unsigned)le << 23))
-                                        : __uint_as_float(sign);
+    unsigned long long b = (unsigned long long)__double_as_longlong(d);
+    unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+    int E = (int)((b >> 52) & 0x7ff);
+    unsigned long long M = (b & 0xfffffffffffffull) | (1ull << 52);  // 53-bit significand
+    unsigned long long H = (M + (1ull << 28)) >> 29;                 // rounded to 24 bits (may be 2^24)
+    long long r = (long long)M - (long long)(H << 29);               // |r| <= 2^28, exact remainder
+    int e = E - 1023 - shift;                                         // unbiased exponent after scaling
+    // hi = H * 2^(e - 23): float bits, the carry of H = 2^24 moves into the exponent
+    unsigned hib = sign | (unsigned)((e + 127) << 23) + (unsigned)(H - (1ull << 23));
+    float hi = (e + 127 > 0 && E != 0) ? __uint_as_float(hib) : 0.0f;
+    // lo = r * 2^(e - 52)
+    float lo = __int2float_rn((int)r);
+    int le = e - 52 + 127;
+    lo = (le > 0 && E != 0) ? lo * __uint_as_float((unsigned)le << 23) : 0.0f;
+    lo = sign ? -lo : lo;
     if (E == 0x7ff) return {__int_as_float(0x7fc00000), 0.0f};  // inf or NaN sample: NaN coefficients
     return {hi, lo};
 }

@@ -16,7 +16,7 @@ namespace rd {
 // so the line lies at 40 polynomials per SM (mixed, from degree 3) and at 8
 // (plain, from degree 6: its FP64 instructions cost the same for one active
 // lane as for 32). Degree 9, the first with 16 lanes per polynomial, has the least
-// to gain; with the compensated polish it ends earlier (complex64 4855 64.3 / 74.5,
+// to gain; with the compensated polish it ends earlier (complex64 4855 68.3 / 78.4,
 // 5923 79.4 / 74.4).
 bool group_takes(int degree, int64_t n, bool mixed, bool compensated)
 {
