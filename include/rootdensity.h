@@ -279,7 +279,8 @@ int rd_pointer_is_device_accessible(const void *p);
  * everything before and after it. The first call on a device from a host thread
  * creates the helper streams and their events; make that call outside capture.
  * (With the launch shape open -- no tuning, no shape in params -- a small batch
- * is solved without bins, in 3 launches on `stream` alone; a
+ * is solved without bins, in 3 launches on `stream` alone, and one of the next
+ * sizes up in 11 to 13, the degrees counted on the device choosing the form; a
  * degree whose tuning entries are all 0 keeps its shape open.) */
 typedef struct {
     /* Launch shape of each degree bin's solve kernel, indexed by the degree

@@ -25,13 +25,33 @@ bool group_takes(int degree, int64_t n, bool mixed, bool compensated)
     return degree >= 3 && n <= (compensated && degree == 9 ? 36 : 40) * sms;
 }
 
-// The same for a packed batch of mixed degrees, which this solver takes in
-// one launch after the count, where the degree bins are twelve kernels side by
-// side, as long as the slowest warp of them. Measured (us, degrees 2..12,
-// complex128, group / bins): mixed 3001 87 / 250, 8000 148 / 290, 16000 236 / 331,
-// 20000 279 / 335, 24000 321 / 341, 30000 383 / 333 (compensated 20000 280 / 296,
-// 24000 320 / 296); plain 2000 1319 / 2172, 4000 2354 / 2351, 8000 4207 / 2587.
-bool uneven_group_takes(int64_t n, bool mixed) { return n <= (int64_t)(mixed ? 144 : 24) * rd_sm_count_cached(); }
+// The same for a packed batch, which this solver takes in one launch after the
+// count, where the degree bins are twelve kernels side by side, as long as the
+// slowest warp of them. What decides is how the degrees are spread, which only
+// the device knows: half-empty kernels lose to the groups up to 144 polynomials
+// per SM, one well-filled kernel of degree 5 and up wins from 56 on (us, group /
+// bins):
+//   degrees 2..12   fp64 8000 140 / 279   14,000 204 / 289   21,000 278 / 299
+//                   df   8000 138 / 229   14,000 206 / 256   21,000 280 / 257
+//   9..12           fp64 14,000 242 / 318  21,000 337 / 336   df 14,000 244 / 264
+//   degree 9        fp64 14,000 175 / 154  21,000 244 / 152   df  8,000 122 / 117  12,000 152 / 119
+//   degree 12       fp64 14,000 260 / 267  21,000 370 / 268   df 12,000 228 / 207
+//   degree 6        fp64 17,000 121 / 128  21,000 142 / 129   df 14,000 103 / 97   21,000 142 / 97
+//   plain           2..12 2000 1319 / 2172, 4000 2354 / 2351; degree 8 3600 1314 / 1060
+// so up to 88 per SM (compensated 56, plain 16) the groups, from 144 (128, 24) the
+// bins; in between the groups, but for a degree with more than a third of the batch
+// from 7 up, above 104 (80, plain always) per SM from 5 up. The launches of the
+// bins that may be asked cost a batch of degrees 2..12 2 to 5 % there, one of
+// degrees 1..4 13 to 20 us of host time.
+UnevenForm uneven_form(int64_t n, bool mixed, bool compensated)
+{
+    const int64_t sms = rd_sm_count_cached();
+    const int sure = !mixed ? 16 : (compensated ? 56 : 88), high = !mixed ? 16 : (compensated ? 80 : 104),
+              most = !mixed ? 24 : (compensated ? 128 : 144);
+    if (n <= sure * sms) return {UnevenForm::group, 0};
+    if (n <= most * sms) return {UnevenForm::ask, n <= high * sms ? 7 : 5};
+    return {UnevenForm::bins, 1};
+}
 
 template <int G, typename In, int MODE>
 static int launch_group_n(int degree, const SolveArgs &a, cudaStream_t st)
@@ -60,23 +80,23 @@ int launch_group(int degree, rd_dtype dt, bool mixed, const SolveArgs &a, cudaSt
 
 template <typename In>
 static int launch_uneven_group_mode(const SolveArgs &a, const UnevenArgs &U, const UnevenHeader *hdr, bool mixed,
-                                    cudaStream_t st)
+                                    bool asked, cudaStream_t st)
 {
     const unsigned grid = (unsigned)((U.n + 1) / 2);
     if (!mixed)
-        uneven_group_kernel<In, MODE_PLAIN><<<grid, GROUP_BLOCK, 0, st>>>(a, U, hdr);
+        uneven_group_kernel<In, MODE_PLAIN><<<grid, GROUP_BLOCK, 0, st>>>(a, U, hdr, asked);
     else if (a.polish_mode == RD_POLISH_DF)
-        uneven_group_kernel<In, MODE_MIXED_DF><<<grid, GROUP_BLOCK, 0, st>>>(a, U, hdr);
+        uneven_group_kernel<In, MODE_MIXED_DF><<<grid, GROUP_BLOCK, 0, st>>>(a, U, hdr, asked);
     else
-        uneven_group_kernel<In, MODE_MIXED_FP64><<<grid, GROUP_BLOCK, 0, st>>>(a, U, hdr);
+        uneven_group_kernel<In, MODE_MIXED_FP64><<<grid, GROUP_BLOCK, 0, st>>>(a, U, hdr, asked);
     return rd_check_launch("uneven_group_kernel");
 }
 
 int launch_uneven_group(const SolveArgs &a, rd_dtype dt, const UnevenArgs &U, const UnevenHeader *hdr, bool mixed,
-                        cudaStream_t st)
+                        bool asked, cudaStream_t st)
 {
-    return dt == RD_C64 ? launch_uneven_group_mode<float2>(a, U, hdr, mixed, st)
-                        : launch_uneven_group_mode<double2>(a, U, hdr, mixed, st);
+    return dt == RD_C64 ? launch_uneven_group_mode<float2>(a, U, hdr, mixed, asked, st)
+                        : launch_uneven_group_mode<double2>(a, U, hdr, mixed, asked, st);
 }
 
 }  // namespace rd

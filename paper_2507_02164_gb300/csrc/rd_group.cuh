@@ -438,14 +438,17 @@ struct DirectMap : ClipFromArrays {
 };
 
 template <typename In, int MODE>
-__global__ void __launch_bounds__(GROUP_BLOCK) uneven_group_kernel(SolveArgs A, UnevenArgs U, const UnevenHeader *hdr)
+__global__ void __launch_bounds__(GROUP_BLOCK) uneven_group_kernel(SolveArgs A, UnevenArgs U, const UnevenHeader *hdr,
+                                                                   bool asked)
 {
+    const unsigned degrees = asked ? hdr->direct : ~0u;  // (0: the ranges overlap, nothing is solved)
+    if (!degrees) return;
     using T = typename std::conditional<MODE != MODE_PLAIN, float, double>::type;
     constexpr int G = 16, P = 32 / G;
     __shared__ GroupMem<T> mem[P];
     __shared__ unsigned long long acc[ST_WORDS];
     const CtaStats S = stats_begin(acc, A.stats);
-    int64_t total = 0;
+    int64_t total = 0;  // (asked: at most what the scan has checked)
     for (int d = 1; d <= UNEVEN_MAX_DEG; ++d) total += (int64_t)__ldg(hdr->count + d) * (d + 1);
     const bool overflow = total > U.n_coeffs;
     const DirectMap map{{}, U.offsets};
@@ -465,7 +468,8 @@ __global__ void __launch_bounds__(GROUP_BLOCK) uneven_group_kernel(SolveArgs A, 
             S.add(ST_STATUS0 + RD_STATUS_DEGENERATE, mark ? 1u : 0u);
             continue;
         }
-        const bool live = d > 0;
+        const bool live = d > 0 && ((degrees >> d) & 1u);
+        if (!__any_sync(0xffffffffu, live)) continue;
         solve_group<G, T, In, MODE>(A, A.coeffs, live ? __ldg(U.offsets + i) : 0, 1, live ? d : 1, live ? i : 0, live,
                                     map, mem[g], S);
     }

@@ -14,7 +14,8 @@
 // header -> count, then for small batches one kernel that gives every polynomial
 // a group of lanes (rd_group.cu), else scan -> pack -> one persistent solve kernel
 // per degree, largest degree first, each with its own register allocation and
-// its own task queue, on several chains of streams (rd_uneven_bins.cuh).
+// its own task queue, on several chains of streams; in between both are launched
+// and the scan chooses by the degrees that it has counted.
 #include "rd_uneven.cuh"
 
 namespace rd {
@@ -64,8 +65,10 @@ __global__ void __launch_bounds__(256) uneven_count_kernel(UnevenArgs U, UnevenH
 // than n_coeffs coefficients in all, their ranges overlap (offsets that are
 // not monotone) and the bins would not fit the workspace: the batch is then
 // not packed or solved (overflow = 1, every count 0), and the pack kernel
-// marks its solvable polynomials DEGENERATE instead.
-__global__ void uneven_scan_kernel(UnevenHeader *hdr, int64_t n_coeffs)
+// marks its solvable polynomials DEGENERATE instead. ask > 0: only a degree from
+// `ask` up that has more than a third of the solvable polynomials keeps its bin,
+// the others go to the group kernel (direct, count 0, not packed).
+__global__ void uneven_scan_kernel(UnevenHeader *hdr, int64_t n_coeffs, int ask)
 {
     const int lane = threadIdx.x;
     unsigned c = lane < 16 ? hdr->count[lane] : 0u;
@@ -83,14 +86,22 @@ __global__ void uneven_scan_kernel(UnevenHeader *hdr, int64_t n_coeffs)
     }
     const int64_t total = __shfl_sync(0xffffffffu, pe, 31);
     const bool overflow = total > n_coeffs;
+    const uint64_t solvable = __shfl_sync(0xffffffffu, pc, 31);
+    const bool grouped = ask && !overflow && !(lane >= ask && 3 * (uint64_t)c > solvable);
+    const unsigned direct = __ballot_sync(0xffffffffu, grouped);
+    const bool any = __any_sync(0xffffffffu, c && !grouped);
     if (lane < 16) {
         hdr->poly_base[lane] = pc - c;  // exclusive
         hdr->coef_base[lane] = pe - e;
         hdr->cursor[lane] = 0;
         hdr->head[lane] = 0;
-        if (overflow) hdr->count[lane] = 0;
+        if (overflow || grouped) hdr->count[lane] = 0;
     }
-    if (lane == 0) hdr->overflow = overflow ? 1u : 0u;
+    if (lane == 0) {
+        hdr->overflow = overflow ? 1u : 0u;
+        hdr->direct = direct;
+        hdr->nothing = any ? 0u : 1u;
+    }
 }
 
 // Scatter every solvable polynomial into its degree's bin: perm[slot] = its
@@ -108,6 +119,7 @@ __global__ void __launch_bounds__(256) uneven_pack_kernel(UnevenArgs U, const E 
                                                           double *roots, uint8_t *status, rd_stats *stats)
 {
     const int lane = threadIdx.x & 31;
+    if (hdr->nothing) return;
     if (hdr->overflow) {
         const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
         const int64_t warp_id = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -131,6 +143,7 @@ __global__ void __launch_bounds__(256) uneven_pack_kernel(UnevenArgs U, const E 
         return;
     }
     __shared__ unsigned cnt[16], first[16];
+    const unsigned direct = hdr->direct;
     for (int64_t base = (int64_t)blockIdx.x * PACK_POLYS; base < U.n; base += (int64_t)gridDim.x * PACK_POLYS) {
         if (threadIdx.x < 16) cnt[threadIdx.x] = 0;
         __syncthreads();
@@ -141,6 +154,7 @@ __global__ void __launch_bounds__(256) uneven_pack_kernel(UnevenArgs U, const E 
             const int64_t i = base + t * 256 + threadIdx.x;
             bool consistent;
             deg[t] = i < U.n ? checked_degree(U, i, consistent) : -1;
+            if (deg[t] > 0 && ((direct >> deg[t]) & 1u)) deg[t] = -1;
             const unsigned act = __ballot_sync(0xffffffffu, deg[t] > 0);
             if (deg[t] > 0) {
                 const unsigned peers = __match_any_sync(act, deg[t]);
@@ -249,6 +263,14 @@ int uneven_fork(cudaStream_t st, int sides, UnevenFork *out, bool retry)
     return RD_OK;
 }
 
+// The other helper streams wait for what the first one has to do so far.
+static int uneven_follow(const UnevenFork &f)
+{
+    cudaError_t e = cudaEventRecord(f.join[0], f.side[0]);
+    for (int k = 1; k < f.sides && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(f.side[k], f.join[0], 0);
+    return e == cudaSuccess ? RD_OK : rd_set_error(RD_ECUDA, "uneven fork: %s", cudaGetErrorString(e));
+}
+
 int uneven_join(cudaStream_t st, const UnevenFork &f)
 {
     for (int k = 0; k < f.sides; ++k) {
@@ -264,6 +286,22 @@ size_t uneven_workspace_bytes(int64_t n, int64_t n_coeffs, rd_dtype dt)
     if (!uneven_sizes_ok(n, n_coeffs)) return 0;
     return uneven_bytes(n, n_coeffs, dt == RD_C64 ? 8 : 16);
 }
+
+// The chains of the degree bins: the caller's stream and helper streams, forked
+// from it and joined back (under stream capture: parallel graph branches), so that
+// other bins' kernels take over the SMs one bin's kernel leaves while its queue
+// drains (a call that may not fork runs them all on the caller's stream). Bins that
+// do not fill the chip are bound by the slowest warp of each kernel and want all
+// twelve side by side; large ones want few kernels competing. Measured (us, degrees 2..12, complex64,
+// FP64 polish; 2 / 4 / 12 chains): 50,000 680 / 536 / 364, 100,000 706 / 517 / 417,
+// 200,000 852 / 619 / 598, 400,000 1075 / 984 / 1003, 2^22 7865 / 7739 / 8100. Degree
+// d goes to chain d mod the number of chains, launched largest first. (Where the
+// scan decides between the group kernel and the bins, the former has the caller's
+// stream, the packing and the bins that may be asked for, at most two of them with
+// work, three helper streams. Behind one another on one stream the empty ones take
+// 5 us each.)
+constexpr int UNEVEN_ASK_SIDES = 3;
+static int uneven_sides(int64_t n) { return n <= (int64_t)1536 * rd_sm_count_cached() ? UNEVEN_SIDES : 3; }
 
 // Whether the degree bins 4 to 12 (compensated polish 7 to 11) take the split-register solver
 // (rd_solve_split.cuh) where the caller left their launch shapes open. The
@@ -300,7 +338,9 @@ int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const
     const bool in_place = r0 && r0 < c0 + (uint64_t)n_coeffs * (dt == RD_C64 ? 8 : 16) && c0 < r0 + (uint64_t)n_roots * 16;
     bool all_open = true;
     for (int d = 1; d <= UNEVEN_MAX_DEG; ++d) all_open &= open_shape[d];
-    if (all_open && !in_place && uneven_group_takes(n, mixed)) {
+    UnevenForm F{UnevenForm::bins, 1};
+    if (all_open && !in_place) F = uneven_form(n, mixed, a.polish_mode == RD_POLISH_DF);
+    if (F.form == UnevenForm::group) {
         // the first call of a host thread, or after a device reset, makes the helper
         // streams whatever its size, so that a larger batch can be captured after it
         cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
@@ -308,7 +348,7 @@ int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const
             UnevenFork none;
             if ((rc = uneven_fork(st, 0, &none))) return rc;
         }
-        return launch_uneven_group(a, dt, U, L.hdr, mixed, st);
+        return launch_uneven_group(a, dt, U, L.hdr, mixed, false, st);
     }
     int bins_pw[16];
     const bool split = uneven_split_takes(n, mixed, a.polish_mode), df = a.polish_mode == RD_POLISH_DF;
@@ -318,26 +358,46 @@ int launch_uneven(const SolveArgs &a, rd_dtype dt, const uint8_t *degrees, const
         bins_pw[d] = takes ? UNEVEN_SPLIT : pw[d];
     }
     pw = bins_pw;
-    uneven_scan_kernel<<<1, 32, 0, st>>>(L.hdr, n_coeffs);
+    const bool ask = F.form == UnevenForm::ask;
+    uneven_scan_kernel<<<1, 32, 0, st>>>(L.hdr, n_coeffs, ask ? F.lowest : 0);
     if ((rc = rd_check_launch("uneven_scan_kernel"))) return rc;
+    UnevenFork f;
+    f.sides = 0;
+    if (ask && fork && (rc = uneven_fork(st, UNEVEN_ASK_SIDES, &f))) return rc;
+    if (ask) rc = launch_uneven_group(a, dt, U, L.hdr, mixed, true, st);
+    cudaStream_t pack = f.sides ? f.side[0] : st;
     if (dt == RD_C64)
-        uneven_pack_kernel<float2><<<(unsigned)ctas, tb, 0, st>>>(U, reinterpret_cast<const float2 *>(a.coeffs), L.hdr,
-                                                                  L.perm, reinterpret_cast<float2 *>(L.bins), a.roots,
-                                                                  a.status, a.stats);
+        uneven_pack_kernel<float2><<<(unsigned)ctas, tb, 0, pack>>>(U, reinterpret_cast<const float2 *>(a.coeffs), L.hdr,
+                                                                    L.perm, reinterpret_cast<float2 *>(L.bins), a.roots,
+                                                                    a.status, a.stats);
     else
-        uneven_pack_kernel<double2><<<(unsigned)ctas, tb, 0, st>>>(U, reinterpret_cast<const double2 *>(a.coeffs),
-                                                                   L.hdr, L.perm, reinterpret_cast<double2 *>(L.bins),
-                                                                   a.roots, a.status, a.stats);
-    if ((rc = rd_check_launch("uneven_pack_kernel"))) return rc;
-    const int mode = !mixed ? MODE_PLAIN : (a.polish_mode == RD_POLISH_DF ? MODE_MIXED_DF : MODE_MIXED_FP64);
-    if (dt == RD_C64) {
-        if (mode == MODE_PLAIN) return launch_uneven_bins<float2, MODE_PLAIN>(a, L, offsets, block, cps, lanes, pw, fork, st);
-        if (mode == MODE_MIXED_DF) return launch_uneven_bins<float2, MODE_MIXED_DF>(a, L, offsets, block, cps, lanes, pw, fork, st);
-        return launch_uneven_bins<float2, MODE_MIXED_FP64>(a, L, offsets, block, cps, lanes, pw, fork, st);
+        uneven_pack_kernel<double2><<<(unsigned)ctas, tb, 0, pack>>>(U, reinterpret_cast<const double2 *>(a.coeffs),
+                                                                     L.hdr, L.perm, reinterpret_cast<double2 *>(L.bins),
+                                                                     a.roots, a.status, a.stats);
+    if (!rc) rc = rd_check_launch("uneven_pack_kernel");
+    if (!rc && ask && f.sides) rc = uneven_follow(f);
+    if (!rc && !ask && fork) {
+        if ((rc = uneven_fork(st, uneven_sides(n), &f))) return rc;
     }
-    if (mode == MODE_PLAIN) return launch_uneven_bins<double2, MODE_PLAIN>(a, L, offsets, block, cps, lanes, pw, fork, st);
-    if (mode == MODE_MIXED_DF) return launch_uneven_bins<double2, MODE_MIXED_DF>(a, L, offsets, block, cps, lanes, pw, fork, st);
-    return launch_uneven_bins<double2, MODE_MIXED_FP64>(a, L, offsets, block, cps, lanes, pw, fork, st);
+    cudaStream_t chain[UNEVEN_MAX_DEG + 1];
+    for (int d = 1; d <= UNEVEN_MAX_DEG; ++d) {
+        const int k = ask ? (f.sides ? 1 + d % f.sides : 0) : d % (f.sides + 1);  // 0: the caller's stream
+        chain[d] = k ? f.side[k - 1] : st;
+    }
+    const int mode = !mixed ? MODE_PLAIN : (a.polish_mode == RD_POLISH_DF ? MODE_MIXED_DF : MODE_MIXED_FP64);
+    auto bins = [&](auto launch) { return launch(a, L, offsets, block, cps, lanes, pw, F.lowest, chain); };
+    if (rc) {
+    } else if (dt == RD_C64) {
+        if (mode == MODE_PLAIN) rc = bins(launch_uneven_bins<float2, MODE_PLAIN>);
+        else if (mode == MODE_MIXED_DF) rc = bins(launch_uneven_bins<float2, MODE_MIXED_DF>);
+        else rc = bins(launch_uneven_bins<float2, MODE_MIXED_FP64>);
+    } else {
+        if (mode == MODE_PLAIN) rc = bins(launch_uneven_bins<double2, MODE_PLAIN>);
+        else if (mode == MODE_MIXED_DF) rc = bins(launch_uneven_bins<double2, MODE_MIXED_DF>);
+        else rc = bins(launch_uneven_bins<double2, MODE_MIXED_FP64>);
+    }
+    const int rj = f.sides ? uneven_join(st, f) : RD_OK;
+    return rc ? rc : rj;
 }
 
 }  // namespace rd

@@ -18,7 +18,8 @@ struct UnevenHeader {
     uint32_t head[16];       // task queue head of each degree's solve kernel
     uint32_t bad;            // polynomials whose offsets disagree with their degree
     uint32_t overflow;       // 1: the solvable polynomials overlap (sum of (d + 1) > n_coeffs)
-    uint32_t pad[2];
+    uint32_t direct;         // bit d: the group kernel solves degree d, its bin is empty
+    uint32_t nothing;        // 1: nothing to pack, every bin is empty
     int64_t coef_base[16];   // first element of each degree's bin in the bins region
 };
 static_assert(sizeof(UnevenHeader) <= 512, "header must fit its 512-byte slot");
@@ -121,19 +122,27 @@ int launch_uneven_split(int degree, rd_dtype dt, const SolveArgs &a, const Uneve
 constexpr int UNEVEN_SPLIT = -1;  // in launch_uneven_bins' pw[d]
 constexpr int SPLIT_DECLINED = 1;  // launch_solve_split, launch_uneven_split: nothing enqueued, take the one-role kernel
 
-// Small batches: every polynomial by a group of lanes, no bins (rd_group.cu).
+// Small batches: every polynomial by a group of lanes, no bins (rd_group.cu);
+// asked = true: those degrees that the scan kernel has left it (hdr->direct).
 int launch_uneven_group(const SolveArgs &a, rd_dtype dt, const UnevenArgs &U, const UnevenHeader *hdr, bool mixed,
-                        cudaStream_t st);
-bool uneven_group_takes(int64_t n, bool mixed);
+                        bool asked, cudaStream_t st);
+// The form of a packed batch: the degree bins, the group kernel, or both launched
+// and the scan kernel deciding by degree, `lowest` and up (below it always groups).
+struct UnevenForm {
+    enum { bins, group, ask } form;
+    int lowest;
+};
+UnevenForm uneven_form(int64_t n, bool mixed, bool compensated);
 
-// Solve every degree bin of a packed batch (one persistent kernel per
-// degree, largest degree first) with the per-degree launch shapes
-// block[d], cps[d], lanes per polynomial lanes[d] and polish warps pw[d]
-// (> 0: the warp-specialised form, mixed mode, degrees up to 8; UNEVEN_SPLIT:
-// the split-register form, degrees 4 to 12, compensated polish 7 to 11).
+// Solve the degree bins of a packed batch from degree `lowest` up (one persistent
+// kernel per degree, largest degree first, degree d on stream chain[d]) with
+// the per-degree launch shapes block[d], cps[d], lanes per polynomial lanes[d]
+// and polish warps pw[d] (> 0: the warp-specialised form, mixed mode, degrees up
+// to 8; UNEVEN_SPLIT: the split-register form, degrees 4 to 12, compensated
+// polish 7 to 11).
 template <typename In, int MODE>
 int launch_uneven_bins(const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets, const int *block,
-                       const int *cps, const int *lanes, const int *pw, bool fork, cudaStream_t st);
+                       const int *cps, const int *lanes, const int *pw, int lowest, const cudaStream_t *chain);
 
 // rd_roots_uneven's argument checks and launch (rd_abi.cu); fork = false
 // keeps every degree bin on `stream` and makes no helper stream.

@@ -170,34 +170,16 @@ static int launch_degree_bin(const SolveArgs &a, const UnevenLayout &L, const in
                              "uneven_solve_kernel");
 }
 
-// The twelve degree bins run as parallel chains of persistent kernels, forked
-// from the caller's stream onto helper streams and joined back (under stream
-// capture: parallel graph branches), so that other bins' kernels take over the
-// SMs one bin's kernel leaves while its queue drains (fork_bins = false: all on
-// the caller's stream, no helper streams). Degree d goes to chain d mod the
-// number of chains, launched largest first. Bins that do not fill the chip are
-// bound by the slowest warp of each kernel and want all twelve side by side;
-// large ones want few kernels competing. Measured (us, degrees 2..12, complex64,
-// FP64 polish; 2 / 4 / 12 chains): 50,000 680 / 536 / 364, 100,000 706 / 517 / 417,
-// 200,000 852 / 619 / 598, 400,000 1075 / 984 / 1003, 2^22 7865 / 7739 / 8100.
-inline int uneven_sides(int64_t n) { return n <= (int64_t)1536 * rd_sm_count_cached() ? 11 : 3; }
-
 template <typename In, int MODE>
 int launch_uneven_bins(const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets, const int *block,
-                       const int *cps, const int *lanes, const int *pw, bool fork_bins, cudaStream_t st)
+                       const int *cps, const int *lanes, const int *pw, int lowest, const cudaStream_t *chain)
 {
-    UnevenFork f;
-    f.sides = 0;
-    int rc = fork_bins ? uneven_fork(st, uneven_sides(a.n), &f) : RD_OK;
-    if (rc) return rc;
-    const int chains = f.sides + 1;
-    auto chain = [&](int d) { return d % chains ? f.side[d % chains - 1] : st; };
+    int rc = RD_OK;
 #define RD_BIN(D) \
-    if (!rc) rc = launch_degree_bin<D, In, MODE>(a, L, offsets, block[D], cps[D], lanes[D], pw[D], chain(D));
+    if (!rc && D >= lowest) rc = launch_degree_bin<D, In, MODE>(a, L, offsets, block[D], cps[D], lanes[D], pw[D], chain[D]);
     RD_BIN(12) RD_BIN(11) RD_BIN(10) RD_BIN(9) RD_BIN(8) RD_BIN(7) RD_BIN(6) RD_BIN(5) RD_BIN(4) RD_BIN(3) RD_BIN(2) RD_BIN(1)
 #undef RD_BIN
-    const int rj = fork_bins ? uneven_join(st, f) : RD_OK;
-    return rc ? rc : rj;
+    return rc;
 }
 
 }  // namespace rd
@@ -205,6 +187,6 @@ int launch_uneven_bins(const SolveArgs &a, const UnevenLayout &L, const int64_t 
 #define RD_UNEVEN_BINS(IN, MODE)                                                                          \
     namespace rd {                                                                                      \
     template int launch_uneven_bins<IN, MODE>(const SolveArgs &, const UnevenLayout &, const int64_t *, \
-                                              const int *, const int *, const int *, const int *, bool, \
-                                              cudaStream_t);                                            \
+                                              const int *, const int *, const int *, const int *, int,  \
+                                              const cudaStream_t *);                                    \
     }
