@@ -866,7 +866,7 @@ def run_uneven(args, rank: int, world: int, local_rank: int, emit: bool = True):
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     from paper_2507_02164_gb300 import autotune
     tuned = autotune.tune("mixed", degrees=range(2, 13))
-    tuning = autotune.uneven_tuning(tuned)
+    tuning = autotune.uneven_tuning(tuned, n)
 
     def step_body():
         api.hist_clear(hist)
@@ -908,7 +908,7 @@ def run_uneven(args, rank: int, world: int, local_rank: int, emit: bool = True):
     # the same batch and graph with the FP32-pipe compensated polish
     # (RD_POLISH_DF), each bin in the one-role shape the tuner picks for it
     tuned_df = autotune.tune("mixed", degrees=range(2, 13), polish="df")
-    tuning_df = autotune.uneven_tuning(tuned_df)
+    tuning_df = autotune.uneven_tuning(tuned_df, n)
     p_df = api.params("mixed", polish_mode="df")
     hist_df = api.new_hist(W_PIX, H_PIX, dev)
     stats_df = api.new_stats(dev)

@@ -102,7 +102,8 @@ def tune(mode: str = "mixed", dtype=torch.complex64, degrees=range(1, 13), n: in
     re-measured.
     Returns {"degrees": {d: {"lanes", "block", "ctas_per_sm", "polish_warps",
     "ms", "one_role": {"lanes", "block", "ctas_per_sm", "ms"}, "open", "table"}},
-    "seconds": time spent measuring, "probe_polys": n}."""
+    "seconds": time spent measuring, "probe_polys": n, "mode", "polish", "sms": the
+    GPU's SM count}."""
     key = cache_key(mode, dtype, n, polish)
     cache = load(cache_path) if cache_path else {}
     entry = cache.get(key, {}) if not force else {}
@@ -125,20 +126,29 @@ def tune(mode: str = "mixed", dtype=torch.complex64, degrees=range(1, 13), n: in
             json.dump(cache, f, indent=1)
         os.replace(tmp, cache_path)
     per_deg = {str(d): entry[str(d)] for d in degrees}
-    return {"degrees": per_deg, "seconds": spent, "probe_polys": n}
+    return {"degrees": per_deg, "seconds": spent, "probe_polys": n, "mode": mode, "polish": polish,
+            "sms": torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count}
 
 
 UNEVEN_WS_MAX_DEG = 8  # the uneven bins have a warp-specialised form up to this degree
+# The degrees whose open bins take the split-register form, and the polynomials per
+# SM of the whole batch from which they do (uneven_split_takes in csrc/rd_uneven.cu).
+UNEVEN_SPLIT = {"fp64": (range(4, 13), 6144), "df": (range(7, 12), 9216)}
 
 
-def uneven_tuning(result: dict):
-    """rd_uneven_tuning (per degree) from a tune() result: each degree's
-    fastest shape where the bins have it (the warp-specialised form up to
-    degree 8), else its fastest one-role shape; left open (all 0) where the open
-    shape won."""
+def uneven_tuning(result: dict, n: int | None = None):
+    """rd_uneven_tuning (per degree) from a tune() result, for batches of n
+    polynomials: each degree's fastest shape where the bins have it (the
+    warp-specialised form up to degree 8), else its fastest one-role shape. Left
+    open (all 0) where the open shape won and an open bin of such a batch is the
+    form that won: the split-register one, in large mixed batches. (The open forms
+    of uniform batches that the bins lack must not leave them untuned; without n
+    no bin is left open.)"""
+    degrees, per_sm = UNEVEN_SPLIT[result.get("polish", "fp64")]
+    split = result.get("mode") == "mixed" and n is not None and n >= per_sm * result["sms"]
     deg = {}
     for d, e in result["degrees"].items():
-        if e.get("open", {}).get("faster"):
+        if split and int(d) in degrees and e.get("open", {}).get("faster"):
             continue
         if int(d) <= UNEVEN_WS_MAX_DEG and e.get("polish_warps", 0) > 0:
             deg[d] = {"block": e["block"], "ctas_per_sm": 0, "lanes": 1, "polish_warps": e["polish_warps"]}
