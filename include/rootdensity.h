@@ -470,10 +470,12 @@ int rd_field_density(rd_field f, const rd_field_spec *spec, rd_mode mode, const 
  * a set for each polish mode. Two lanes are not a candidate with RD_POLISH_DF.
  * Each shape runs once untimed, then `reps` times (1..15) timed with CUDA
  * events; its time is the median. A shape that cannot be launched (too many
- * registers for the block) is recorded with ms < 0 and skipped. This is the
+ * registers for the block) is recorded with ms < 0 and skipped. The open shape
+ * (every launch field 0), which reaches forms that no explicit shape names, is not
+ * among them: time a call with it too and keep it where it is faster. This is the
  * one entry point that allocates (the probe batch and its histogram, freed
  * before it returns) and synchronises: call it outside any stream capture.
- *   out        host; the fastest shape, and the fastest with polish_warps = 0
+ *   out        host; the fastest explicit shape, and the fastest with polish_warps = 0
  *              (the form the uneven-degree bins run)
  *   table      host array of table_cap entries or NULL; receives every timed
  *              shape (at most table_cap), *table_len their number
@@ -483,7 +485,7 @@ typedef struct {
     float ms;      /* median milliseconds of one rd_roots_density call on the probe, < 0: not launchable */
 } rd_tune_entry;
 typedef struct {
-    rd_tune_entry best;      /* fastest shape overall                                      */
+    rd_tune_entry best;      /* fastest explicit shape                                     */
     rd_tune_entry one_role;  /* fastest shape with polish_warps = 0                         */
     int32_t n_candidates;    /* shapes timed (launchable or not)                           */
     int32_t reserved;
