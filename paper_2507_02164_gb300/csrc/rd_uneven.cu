@@ -18,6 +18,8 @@
 // and the scan chooses by the degrees that it has counted.
 #include "rd_uneven.cuh"
 
+#include <cuda.h>
+
 namespace rd {
 
 int launch_clear(uint32_t *p, int64_t words, cudaStream_t st);
@@ -182,10 +184,43 @@ __global__ void __launch_bounds__(256) uneven_pack_kernel(UnevenArgs U, const E 
 }
 
 namespace {
+// Driver entry points (looked up at run time: the library links the runtime only).
+template <typename F>
+F driver_entry(const char *name)
+{
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess)
+        return nullptr;
+    return reinterpret_cast<F>(p);
+}
+
+// The current context's id, unique for the life of the process (0: none). A
+// device reset gives the next context another one; the handles of the old one may
+// not even be looked at then.
+unsigned long long context_id()
+{
+    static const auto get = driver_entry<CUresult (*)(CUcontext, unsigned long long *)>("cuCtxGetId");
+    unsigned long long id = 0;
+    return get && get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+bool primary_context_active(int dev)
+{
+    static const auto get = driver_entry<CUresult (*)(CUdevice, unsigned *, int *)>("cuDevicePrimaryCtxGetState");
+    unsigned flags = 0;
+    int active = 0;
+    return get && get(dev, &flags, &active) == CUDA_SUCCESS && active;
+}
+
 // The helper streams, the fork event and a join event for each, per device,
-// owned by one host thread and released when that thread exits (errors
-// ignored: at process exit the runtime may already be gone).
+// owned by one host thread and released when that thread exits, unless their
+// context is gone by then (errors ignored: at process exit the runtime may
+// already be gone).
 struct ForkState {
+    int device = -1;
+    unsigned long long context = 0;
     cudaStream_t side[UNEVEN_SIDES] = {};
     cudaEvent_t fork = nullptr, join[UNEVEN_SIDES] = {};
     void release()
@@ -204,7 +239,17 @@ struct ForkState {
             side[k] = nullptr;
         }
     }
-    ~ForkState() { release(); }
+    ~ForkState()
+    {
+        if (!fork) return;
+        int current = 0;
+        if (context_id() == context) {
+            release();
+        } else if (primary_context_active(device) && cudaGetDevice(&current) == cudaSuccess && current != device) {
+            if (cudaSetDevice(device) == cudaSuccess && context_id() == context) release();
+            cudaSetDevice(current);
+        }
+    }
 };
 thread_local ForkState g_fork[64];
 }  // namespace
@@ -217,7 +262,11 @@ static int uneven_handles(ForkState **out)
     if (e != cudaSuccess) return rd_set_error(RD_ECUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
     if (dev < 0 || dev >= 64) return rd_set_error(RD_EUNSUPPORTED, "device index %d above 63", dev);
     ForkState &f = g_fork[dev];
+    const unsigned long long context = context_id();
+    if (f.fork && f.context != context) f.forget();  // made before a device reset
     if (!f.fork) {
+        f.device = dev;
+        f.context = context;
         // all or none: a partial failure releases what it made
         e = cudaEventCreateWithFlags(&f.fork, cudaEventDisableTiming);
         for (int k = 0; k < UNEVEN_SIDES && e == cudaSuccess; ++k) {
@@ -236,25 +285,15 @@ static int uneven_handles(ForkState **out)
     return RD_OK;
 }
 
-int uneven_fork(cudaStream_t st, int sides, UnevenFork *out, bool retry)
+int uneven_fork(cudaStream_t st, int sides, UnevenFork *out)
 {
     ForkState *state = nullptr;
     int rc = uneven_handles(&state);
     if (rc) return rc;
     ForkState &f = *state;
-    cudaError_t e;
-    e = cudaEventRecord(f.fork, st);
+    cudaError_t e = sides ? cudaEventRecord(f.fork, st) : cudaSuccess;
     for (int k = 0; k < sides && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(f.side[k], f.fork, 0);
-    if (e != cudaSuccess) {
-        // handles made before a cudaDeviceReset are gone (the runtime answers with
-        // either code): forget them (they cannot be destroyed any more) and make
-        // new ones, once
-        if ((e != cudaErrorInvalidResourceHandle && e != cudaErrorContextIsDestroyed) || retry)
-            return rd_set_error(RD_ECUDA, "uneven fork: %s", cudaGetErrorString(e));
-        cudaGetLastError();
-        f.forget();
-        return uneven_fork(st, sides, out, true);
-    }
+    if (e != cudaSuccess) return rd_set_error(RD_ECUDA, "uneven fork: %s", cudaGetErrorString(e));
     out->sides = sides;
     for (int k = 0; k < sides; ++k) {
         out->side[k] = f.side[k];

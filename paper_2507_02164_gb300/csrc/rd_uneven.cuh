@@ -102,7 +102,7 @@ struct UnevenFork {
     cudaStream_t side[UNEVEN_SIDES];
     cudaEvent_t join[UNEVEN_SIDES];
 };
-int uneven_fork(cudaStream_t st, int sides, UnevenFork *out, bool retry = false);
+int uneven_fork(cudaStream_t st, int sides, UnevenFork *out);
 int uneven_join(cudaStream_t st, const UnevenFork &f);
 
 // The split-register solver hands tasks of 32 polynomials between warps with
