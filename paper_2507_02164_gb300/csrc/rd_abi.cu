@@ -161,13 +161,17 @@ bool shape_open(const rd_params &p)
 //    9           144 / 148  165 / 172  216 / 233  240 / 265  325 / 364  625 / 735  1069 / 1305
 //   10           176 / 187  204 / 213  265 / 297  296 / 339  392 / 458  754 / 929  1286 / 1621
 //   11           226 / 246  268 / 261  349 / 374  396 / 394  526 / 546  997 / 1101 1672 / 1911
-// (25,000: 9 100 / 92, 11 141 / 138).
+// (25,000: 9 100 / 92, 11 141 / 138; 52,781, where 128 threads fill the SMs evenly,
+// 9 156 / 151, complex128 174 / 163: left out.)
 // (Only with sweep bounds that its waits allow for: split_waits_ok.)
 bool split_takes(int degree, rd_dtype dtype, int64_t n, bool mixed, const rd_params &p)
 {
     if (!mixed || degree < 4 || !rd::split_waits_ok(degree, p.max_iters, p.fixed_sweeps)) return false;
     const int64_t per_sm = n / rd_sm_count_cached();
-    if (p.polish_mode == RD_POLISH_DF) return degree >= 7 && degree <= 11 && per_sm >= (degree == 7 ? 1536 : (degree == 8 ? 640 : 256));
+    if (p.polish_mode == RD_POLISH_DF) {
+        if (degree == 9 && per_sm >= 344 && per_sm < 352) return false;
+        return degree >= 7 && degree <= 11 && per_sm >= (degree == 7 ? 1536 : (degree == 8 ? 640 : 256));
+    }
     if (degree == 4) return dtype == RD_C64 && per_sm >= 640;
     return per_sm >= (degree <= 6 ? 576 : (degree <= 8 ? 352 : 224));
 }
@@ -198,24 +202,25 @@ bool pool_takes(int degree, int64_t n)
 //     compensated polish, which does not live on the FP64 unit, up to two warps
 //     per sub-partition (8 complex128 30,000 90 / 86), degree 12 always (100,003
 //     543 / 534, 300,007 1462 / 1422).
-//   up to twelve warps per SM, a batch that all but fills its CTAs of four or of
-//     two warps on every SM: single-warp CTAs then land unevenly on the
-//     sub-partitions (32 / 64 / 128 threads): 35,462, 7.3 warps, plain 12 3697 / 3505 /
-//     3501, plain 2 18.9 / 17.2 / 17.1; 29,067, 6.0, plain 9 (complex128) 1.13 / 1.00
-//     / 1.30 of the best; 52,781, 10.9, compensated 9 (complex128) 170 / 170 / 165.
+//   up to eight warps per SM (compensated polish: twelve), a batch that all but
+//     fills its CTAs of four or of two warps on every SM: single-warp CTAs then land
+//     unevenly on the sub-partitions (32 / 64 / 128 threads): 35,462, 7.3 warps,
+//     mixed 6 1.03 / 1.00 / 1.00 of the best, plain 12 3697 / 3505 / 3501, plain 2 18.9 /
+//     17.2 / 17.1 (3 to 11 gain nothing from 128); 29,067, 6.0, plain 9 (complex128)
+//     1.13 / 1.00 / 1.30; 52,781, 10.9, compensated 5 (complex128) 49.9 / 49.8 / 48.2.
 //   compensated polish, twelve to 32 warps per SM: two warps per CTA: 116,927
 //     degree 2 16.4 / 15.2 / 15.2, 78,559 degree 3 29.0 / 28.1 / 28.3.
 //   compensated polish, degrees 5 and 6, many waves: 256 threads: degree 6 300,000
 //     265 against 278, 2^20 904 against 973, 2^19 448 against 470.
 void open_shape(rd_params &p, int degree, int64_t n, bool mixed)
 {
-    const int64_t sms = rd_sm_count_cached(), per_sm = n / sms;
+    const int64_t sms = rd_sm_count_cached(), per_sm = (n + sms - 1) / sms;
     const bool df = mixed && p.polish_mode == RD_POLISH_DF;
     p.block = 32;
     if (n <= (df ? 256 : 128) * sms) {
         if (mixed || n > 96 * sms) p.block = 128;
-    } else if (n <= 384 * sms) {
-        if (per_sm % 128 == 0 || per_sm % 128 >= 88)
+    } else if (n <= (df ? 384 : 256) * sms) {
+        if ((mixed || degree <= 2 || degree == 12) && (per_sm % 128 == 0 || per_sm % 128 >= 88))
             p.block = 128;
         else if (!df && (per_sm % 64 == 0 || per_sm % 64 >= 56))
             p.block = 64;
