@@ -87,9 +87,11 @@ __device__ __forceinline__ void adjoint_term(cx<T> &g, cx<T> &pw, cx<T> u, cx<T>
 
 // One thread per polynomial. Bound by the FP64 pipe (complex128: about 80
 // operations per root of degree 6) or by memory (complex64: 304 bytes per
-// polynomial, all loads issued before the first use). 2^20 polynomials of
-// degree 6: complex128 873 us (1,066 with 110 operations per root), complex64
-// 58 us, 5.5 TB/s (62).
+// polynomial). All loads are issued before the first use: at degree 12 complex128
+// holds 244 registers for it where loads in the loop hold 144, which the FP64 pipe
+// does not notice. 2^20 polynomials of degree 6: complex128 873 us (1,066 with 110
+// operations per root, loads in the loop), complex64 58 us, 5.5 TB/s (62); 2^18,
+// complex128: degree 3 74.5 (92.8), 8 381 (460), 12 797 (948).
 template <int N, typename T>
 __global__ void __launch_bounds__(256) backward_kernel(const void *coeffs, const double2 *__restrict__ roots,
                                                        const double2 *__restrict__ grad_roots, void *grad_coeffs,
