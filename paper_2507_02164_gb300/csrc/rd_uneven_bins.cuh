@@ -125,17 +125,26 @@ static int launch_uneven_ws(const SolveArgs &a, const UnevenLayout &L, const int
 
 int lanes_for(int degree, bool mixed, int polish_mode, int requested);
 
-template <typename K>
-static int launch_persistent(K kern, const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets, int block,
+// The occupancy maximum is asked for once per kernel, device and block size (0.2 us
+// each time, of about 5 us of host time per bin).
+template <auto KERN>
+static int launch_persistent(const SolveArgs &a, const UnevenLayout &L, const int64_t *offsets, int block,
                              int ctas_per_sm, cudaStream_t st, const char *what)
 {
-    int per_sm = ctas_per_sm;
+    static std::atomic<int> known[64][9];
+    int per_sm = ctas_per_sm, dev = 0;
     if (per_sm <= 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, 0) != cudaSuccess || per_sm < 1)
-            per_sm = 1;
+        const bool keep = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && block <= 256;
+        per_sm = keep ? known[dev][block / 32].load(std::memory_order_relaxed) : 0;
+        if (per_sm <= 0) {
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, KERN, block, 0) != cudaSuccess || per_sm < 1)
+                per_sm = 1;
+            else if (keep)
+                known[dev][block / 32].store(per_sm, std::memory_order_relaxed);
+        }
     }
     int grid = per_sm * rd_sm_count_cached();
-    kern<<<grid, block, 0, st>>>(a, L.hdr, L.perm, L.bins, offsets);
+    KERN<<<grid, block, 0, st>>>(a, L.hdr, L.perm, L.bins, offsets);
     return rd_check_launch(what);
 }
 
@@ -154,7 +163,7 @@ static int launch_degree_bin(const SolveArgs &a, const UnevenLayout &L, const in
     }
     if constexpr (N >= 2 && MODE != MODE_MIXED_DF) {
         if (lanes_for(N, MODE != MODE_PLAIN, a.polish_mode, lanes) == 2)
-            return launch_persistent(uneven_solve2_kernel<N, In, MODE>, a, L, offsets, block, ctas_per_sm, st,
+            return launch_persistent<uneven_solve2_kernel<N, In, MODE>>(a, L, offsets, block, ctas_per_sm, st,
                                      "uneven_solve2_kernel");
     }
     // At most eight warps per SM whatever the bin's share of the batch: free
@@ -163,10 +172,10 @@ static int launch_degree_bin(const SolveArgs &a, const UnevenLayout &L, const in
     // 34,000 166 / 133, 50,000 167 / 210).
     if constexpr (solve_twelve_warps(N, MODE)) {
         if (a.n > 256 * (int64_t)rd_sm_count_cached())
-            return launch_persistent(uneven_solve_kernel<N, In, MODE, true>, a, L, offsets, block, ctas_per_sm, st,
+            return launch_persistent<uneven_solve_kernel<N, In, MODE, true>>(a, L, offsets, block, ctas_per_sm, st,
                                      "uneven_solve_kernel");
     }
-    return launch_persistent(uneven_solve_kernel<N, In, MODE, false>, a, L, offsets, block, ctas_per_sm, st,
+    return launch_persistent<uneven_solve_kernel<N, In, MODE, false>>(a, L, offsets, block, ctas_per_sm, st,
                              "uneven_solve_kernel");
 }
 
